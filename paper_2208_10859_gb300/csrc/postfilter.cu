@@ -16,9 +16,9 @@
 //     (dy, dx) is the row slot of dy shifted by dx pixels: only the
 //     descriptor's start address changes (SBO = 128 bytes, LBO = one column).
 //   forward / input gradient, 1 input channel: K = the 9 taps (padded to 16).
-//   weight gradient, 32 -> 32: D[tap, ci][co] = sum over pixels of
-//     input[p + tap][ci] * dZ[p][co]: M = 288 rows (+ one row of ones that
-//     yields the bias gradient), N = 32, K = pixels in chunks of 64.
+//   weight gradient, 32 -> 32: D[dy, ci][dx, co] = sum over pixels of
+//     input[p + (dy, dx)][ci] * dZ[p][co]: M = (dy, ci), N = co, K = pixels,
+//     one accumulator per dx, both operands read channel-major.
 //   The input gradient of a layer is a forward convolution of the output
 //   gradient with the spatially flipped, channel-transposed weights; the
 //   ReLU of the layer below gates it in the epilogue.
@@ -323,95 +323,105 @@ __global__ void __launch_bounds__(128) k_conv_in1(ConvArgs a) {
     if (warp == 0) umma::tmem_free<32>(tmem);
 }
 
-// Weight gradient of a 32 -> 32 layer on the tensor cores.  Per chunk of 64
-// pixels of one image row: A[(tap, ci)][p] = act[p + tap][ci] (288 rows, row
-// 288 = 1 for the bias gradient, rows up to 383 zero), B[co][p] = dz[p][co],
-// both transposed into K-major tiles in shared memory; three M-tiles of 128
-// rows accumulate in TMEM over all chunks of the CTA, then are added to the
-// global gradient.
-constexpr int kWChunk = 64;
-constexpr int kWRows = 384;
-constexpr int kWAStep = kWRows * 32;
-constexpr int kWA = 4 * kWAStep;
-constexpr int kWB = 4 * kStep32;
-constexpr int kWAct = 3 * (kWChunk + 2) * 64;
-constexpr int kWDz = kWChunk * 64;
-constexpr int kWSmem = kWA + kWB + kWAct + kWDz;
+// Weight gradient of a 32 -> 32 layer on the tensor cores:
+// dW[tap][ci][co] = sum over pixels of act[p + tap][ci] dz[p][co].  The sum
+// runs over pixels, so both operands are read with their channels along the
+// MMA's M or N and pixels along K: exactly how the channel-last rows lie in
+// shared memory as 8-channel columns (16 bytes a pixel), with the descriptor's
+// "MN-major" form; nothing is transposed.  A tile is kWRowsT rows x 128 pixels
+// of dz with the kWRowsT + 2 rows of act around them.  For row y and shift dx,
+// A starts at act row y - 1, pixel dx: consecutive row slots continue the
+// 8-channel columns, so its M = 128 holds (dy, ci) for dy = 0..2 (the fourth
+// row's products land in accumulator rows that are never read).  The three dx
+// accumulate in three 32-column TMEM ranges over all tiles of the CTA, which
+// adds them to the global gradient once at its end, in the gradient's order.
+// The bias gradient is summed from the dz rows in shared memory meanwhile.
+//
+// Bound: the MMAs' reads of A (4 KB per 16 pixels and dx) and the 128 bytes
+// per pixel from HBM, about 20 us each for 16 x 256^2 pixels; two CTAs per SM
+// so that one's loads run under the other's MMAs.  Measured 79 us; the form
+// with both operands transposed through shared memory by the threads 434 us.
+constexpr int kWRowsT = 4;                              // dz rows per tile
+constexpr int kWThreads = 256;
+constexpr int kWAct = (kWRowsT + 3) * kSlot;            // kWRowsT + 2 rows, one more that the last M reads
+constexpr int kWDz = kWRowsT * kSlot;                   // dz rows in the same layout (pixels 0..127)
+constexpr int kWSmem = kWAct + kWDz;
+static_assert(kC * kC * 9 * 4 <= kWSmem, "the gradient is staged in the operand buffers");
 
-__global__ void __launch_bounds__(128) k_wgrad_mid(const bf16 *__restrict__ act, const bf16 *__restrict__ dz,
-                                                   int n, int h, int w, float *dW, float *db, int *err) {
+__device__ __forceinline__ void cp_async16(uint8_t *dst, const void *src, bool fill) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(umma::smem_addr(dst)), "l"(src),
+                 "r"(fill ? 16 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restrict__ act, const bf16 *__restrict__ dz,
+                                                           int n, int h, int w, float *dW, float *db, int *err) {
     extern __shared__ __align__(128) uint8_t sm[];
-    uint8_t *sA = sm, *sB = sm + kWA, *sAct = sB + kWB, *sDz = sAct + kWAct;
+    uint8_t *sAct = sm, *sDz = sm + kWAct;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
+    __shared__ float sBias[kC];
     const int tid = threadIdx.x, warp = tid >> 5;
-    // rows 288..383 of every K-step: ones (row 288), zeros
-    for (int i = tid; i < 4 * 96 * 8; i += 128) {
-        const int s = i / (96 * 8), r = 288 + (i / 8) % 96, kp = i % 8;
-        const float one = r == 288 ? 1.f : 0.f;
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn(one, one);
-        *reinterpret_cast<__nv_bfloat162 *>(sA + s * kWAStep + umma::kstep_offset(r, 2 * kp)) = b2;
-    }
     if (tid == 0) umma::mbar_init(&mbar, 1);
+    if (tid < kC) sBias[tid] = 0.f;
     if (warp == 0) umma::tmem_alloc<128>(&tmem_base);
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
-    const uint32_t idesc = umma::idesc_bf16(128, 32);
-    const int xchunks = (w + kWChunk - 1) / kWChunk;
-    const int total = n * h * xchunks;
+    const uint32_t idesc = umma::idesc_bf16(128, 32) | umma::kAMnMajor | umma::kBMnMajor;
+    const int tx = (w + kTilePx - 1) / kTilePx, ty = (h + kWRowsT - 1) / kWRowsT;
+    const int total = n * tx * ty;
     uint32_t phase = 0;
     bool first = true, ok = true;
-    for (int ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int xc = ch % xchunks, y = (ch / xchunks) % h, img = ch / (xchunks * h);
-        const int x0 = xc * kWChunk;
-        for (int i = tid; i < 3 * (kWChunk + 2) * 4; i += 128) {
-            const int q = i & 3, px = (i >> 2) % (kWChunk + 2), dy = (i >> 2) / (kWChunk + 2);
-            const int yy = y + dy - 1, xx = x0 - 1 + px;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (yy >= 0 && yy < h && xx >= 0 && xx < w)
-                v = __ldg(reinterpret_cast<const uint4 *>(act + (((size_t)img * h + yy) * w + xx) * kC + q * 8));
-            *reinterpret_cast<uint4 *>(sAct + (dy * (kWChunk + 2) + px) * 64 + q * 16) = v;
+    float bsum[8] = {};   // channels 8 (tid & 3) ..
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const int x0 = (it % tx) * kTilePx, y0 = ((it / tx) % ty) * kWRowsT, img = it / (tx * ty);
+        const int rows = min(kWRowsT, h - y0);
+        const int steps = (min(kTilePx, w - x0) + 15) / 16;   // K-steps of 16 pixels
+        const int apx = 16 * steps + 2;
+        for (int i = tid; i < (rows + 2) * apx * 4; i += kWThreads) {
+            const int q = i & 3, px = (i >> 2) % apx, r = (i >> 2) / apx;
+            const int yy = y0 + r - 1, xx = x0 - 1 + px;
+            const bool in = yy >= 0 && yy < h && xx >= 0 && xx < w;
+            cp_async16(sAct + r * kSlot + q * kLbo + px * 16,
+                       in ? act + (((size_t)img * h + yy) * w + xx) * kC + q * 8 : act, in);
         }
-        for (int i = tid; i < kWChunk * 4; i += 128) {
-            const int q = i & 3, px = i >> 2, xx = x0 + px;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (xx < w) v = __ldg(reinterpret_cast<const uint4 *>(dz + (((size_t)img * h + y) * w + xx) * kC + q * 8));
-            *reinterpret_cast<uint4 *>(sDz + px * 64 + q * 16) = v;
+        for (int i = tid; i < rows * steps * 64; i += kWThreads) {
+            const int q = i & 3, px = (i >> 2) % (16 * steps), r = (i >> 2) / (16 * steps);
+            const int yy = y0 + r, xx = x0 + px;
+            const bool in = xx < w;
+            cp_async16(sDz + r * kSlot + q * kLbo + px * 16,
+                       in ? dz + (((size_t)img * h + yy) * w + xx) * kC + q * 8 : dz, in);
         }
-        __syncthreads();
-        // transpose into the K-major operands: pairs of pixels per store
-        for (int i = tid; i < 288 * (kWChunk / 2); i += 128) {
-            const int m = i % 288, kp = i / 288, k = 2 * kp;
-            const int tap = m >> 5, ci = m & 31, dy = tap / 3, dx = tap % 3;
-            const bf16 *row = reinterpret_cast<const bf16 *>(sAct + (dy * (kWChunk + 2) + k + dx) * 64) + ci;
-            __nv_bfloat162 b2;
-            b2.x = row[0];
-            b2.y = row[32];
-            *reinterpret_cast<__nv_bfloat162 *>(sA + (k >> 4) * kWAStep + umma::kstep_offset(m, k & 15)) = b2;
-        }
-        for (int i = tid; i < 32 * (kWChunk / 2); i += 128) {
-            const int co = i & 31, kp = i >> 5, k = 2 * kp;
-            const bf16 *col = reinterpret_cast<const bf16 *>(sDz + k * 64) + co;
-            __nv_bfloat162 b2;
-            b2.x = col[0];
-            b2.y = col[32];
-            *reinterpret_cast<__nv_bfloat162 *>(sB + (k >> 4) * kStep32 + umma::kstep_offset(co, k & 15)) = b2;
-        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
         umma::fence_smem_to_async();
         umma::fence_before_sync();
         __syncthreads();
         umma::fence_after_sync();
         if (tid == 0) {
-            const uint32_t a0 = umma::smem_addr(sA), b0 = umma::smem_addr(sB);
+            const uint32_t a0 = umma::smem_addr(sAct), b0 = umma::smem_addr(sDz);
 #pragma unroll 1
-            for (int s = 0; s < 4; ++s)
+            for (int r = 0; r < rows; ++r)
+#pragma unroll 1
+                for (int s = 0; s < steps; ++s) {
+                    const uint64_t bd = umma::desc(b0 + r * kSlot + s * 256, 128, kLbo);
 #pragma unroll
-                for (int mt = 0; mt < 3; ++mt)
-                    umma::mma(tmem + 32 * mt, umma::desc(a0 + s * kWAStep + mt * 4096, 128, 256),
-                              umma::desc(b0 + s * kStep32, 128, 256), idesc, !(first && s == 0));
+                    for (int dx = 0; dx < 3; ++dx)
+                        umma::mma(tmem + 32 * dx, umma::desc(a0 + r * kSlot + s * 256 + dx * 16, 128, kLbo), bd, idesc,
+                                  !(first && r == 0 && s == 0));
+                }
             umma::commit(&mbar);
+        }
+        for (int i = tid; i < rows * steps * 64; i += kWThreads) {
+            const int px = (i >> 2) % (16 * steps), r = (i >> 2) / (16 * steps);
+            const uint4 v = *reinterpret_cast<const uint4 *>(sDz + r * kSlot + (tid & 3) * kLbo + px * 16);
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                bsum[2 * e] += __uint_as_float(u[e] << 16);
+                bsum[2 * e + 1] += __uint_as_float(u[e] & 0xffff0000u);
+            }
         }
         const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase));
         phase ^= 1;
@@ -423,18 +433,28 @@ __global__ void __launch_bounds__(128) k_wgrad_mid(const bf16 *__restrict__ act,
         first = false;
     }
     if (!first && ok) {
+        // the accumulators, reordered to the gradient's [co][ci][tap] in the
+        // operand buffers (the MMAs have completed), then one coalesced pass
         umma::fence_after_sync();
-        for (int mt = 0; mt < 3; ++mt) {
+        float *out = reinterpret_cast<float *>(sm);
+        const int m = (warp & 3) * 32 + (tid & 31), dy = m >> 5, ci = m & 31;
+        for (int dx = warp >> 2; dx < 3; dx += kWThreads / 128) {
             float v[32];
-            umma::ld32(tmem + 32 * mt + ((uint32_t)(warp * 32) << 16), v);
-            const int m = mt * 128 + warp * 32 + (tid & 31);
-            if (m < 288) {
-                const int tap = m >> 5, ci = m & 31;
-                for (int co = 0; co < 32; ++co) atomicAdd(dW + (co * kC + ci) * 9 + tap, v[co]);
-            } else if (m == 288) {
-                for (int co = 0; co < 32; ++co) atomicAdd(db + co, v[co]);
-            }
+            umma::ld32(tmem + 32 * dx + ((uint32_t)((warp & 3) * 32) << 16), v);
+            if (dy < 3)
+#pragma unroll
+                for (int co = 0; co < 32; ++co) out[(co * kC + ci) * 9 + dy * 3 + dx] = v[co];
         }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            float v = bsum[e];
+#pragma unroll
+            for (int o = 4; o < 32; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if ((tid & 31) < 4) atomicAdd(&sBias[8 * (tid & 3) + e], v);
+        }
+        __syncthreads();
+        for (int i = tid; i < kC * kC * 9; i += kWThreads) atomicAdd(dW + i, out[i]);
+        if (tid < kC) atomicAdd(db + tid, sBias[tid]);
     }
     umma::fence_before_sync();
     __syncthreads();
@@ -442,78 +462,82 @@ __global__ void __launch_bounds__(128) k_wgrad_mid(const bf16 *__restrict__ act,
 }
 
 // Weight gradients of the first (1 -> 32) and last (32 -> 1) layers on CUDA
-// cores: thread j of 320 accumulates one (channel, tap) product over the
-// chunks of its CTA (tap 9 = the bias).
-__global__ void __launch_bounds__(320) k_wgrad_edge(const float *__restrict__ plane, const bf16 *__restrict__ act,
-                                                    int first_layer, int n, int h, int w, float *dW, float *db) {
-    __shared__ float sP[3 * (kWChunk + 2)];       // first layer: input luma rows
-    __shared__ float sG[kWChunk];                 // last layer: dz plane
-    __shared__ __align__(16) bf16 sT[3 * (kWChunk + 2) * kC];   // 32-channel tensor rows
-    const int tid = threadIdx.x;
-    const int xchunks = (w + kWChunk - 1) / kWChunk;
-    const int total = n * h * xchunks;
-    float acc = 0.f;
-    // first layer: c = tid % 32 output channel, j = tid / 32 tap (9: bias);
-    // last layer: c = tid % 32 input channel, j = tid / 32 tap (9: bias)
-    const int c = tid & 31, j = tid >> 5;
-    for (int ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const int xc = ch % xchunks, y = (ch / xchunks) % h, img = ch / (xchunks * h);
-        const int x0 = xc * kWChunk;
-        __syncthreads();
-        if (first_layer) {
-            // plane = input luma (3 rows with halo); act = dZ of layer 0 (this row)
-            for (int i = tid; i < 3 * (kWChunk + 2); i += 320) {
-                const int px = i % (kWChunk + 2), dy = i / (kWChunk + 2);
-                const int yy = y + dy - 1, xx = x0 - 1 + px;
-                sP[i] = (yy >= 0 && yy < h && xx >= 0 && xx < w) ? plane[((size_t)img * h + yy) * w + xx] : 0.f;
+// cores, in fp32: G[tap][c] = sum over pixels q of T[q][c] P[q + tap - 1],
+// with T the layer's 32-channel tensor and P its one-channel plane.  First
+// layer: T = dZ, P = the input, tap as is; last layer: T = the input, P = dZ,
+// tap flipped (T[p + tap - 1] P[p] = T[q] P[q - (tap - 1)]).  A half warp walks
+// along a run of kERun pixels, each lane with two channels (one 4-byte load a
+// pixel) and the 3 x 3 window of P sliding in registers: 3 loads and 18 FMAs
+// a pixel, about 25 instructions per two pixels.  66 us for 16 x 256^2
+// pixels; the form staged in shared memory, with two loads per FMA, took 138
+// and 153 us.
+constexpr int kERun = 32;        // pixels per half warp and work item
+constexpr int kEWarps = 8;
+
+__global__ void __launch_bounds__(32 * kEWarps) k_wgrad_edge(const float *__restrict__ plane,
+                                                            const bf16 *__restrict__ act, int first_layer, int n, int h,
+                                                            int w, float *dW, float *db) {
+    __shared__ float sum[kC * 9 + kC];   // [c][tap], then the bias
+    const int tid = threadIdx.x, lane = tid & 31, half = lane >> 4, c = 2 * (lane & 15);
+    for (int i = tid; i < kC * 10; i += 32 * kEWarps) sum[i] = 0.f;
+    __syncthreads();
+    float acc0[9] = {}, acc1[9] = {}, b0 = 0.f, b1 = 0.f;
+    const int runs = (w + 2 * kERun - 1) / (2 * kERun);
+    const int total = n * h * runs;
+    for (int it = blockIdx.x * kEWarps + (tid >> 5); it < total; it += gridDim.x * kEWarps) {
+        const int y = (it / runs) % h, img = it / (runs * h);
+        const int xa = (it % runs) * 2 * kERun + half * kERun;
+        const float *row = plane + ((size_t)img * h + y) * w;
+        const uint32_t *t = reinterpret_cast<const uint32_t *>(act + ((size_t)img * h + y) * w * kC + c);
+        const bool up = y > 0, dn = y + 1 < h;
+        auto load = [&](int x, float (&v)[3]) {
+            const bool in = x >= 0 && x < w;
+            v[0] = in && up ? __ldg(row - w + x) : 0.f;
+            v[1] = in ? __ldg(row + x) : 0.f;
+            v[2] = in && dn ? __ldg(row + w + x) : 0.f;
+        };
+        float p0[3], p1[3];
+        load(xa - 1, p0);
+        load(xa, p1);
+#pragma unroll 4
+        for (int k = 0; k < kERun; ++k) {
+            const int x = xa + k;
+            float p2[3];
+            load(x + 1, p2);
+            const uint32_t u = x < w ? __ldg(t + (size_t)x * (kC / 2)) : 0u;
+            const float t0 = __uint_as_float(u << 16), t1 = __uint_as_float(u & 0xffff0000u);
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                acc0[3 * dy] = fmaf(t0, p0[dy], acc0[3 * dy]);
+                acc1[3 * dy] = fmaf(t1, p0[dy], acc1[3 * dy]);
+                acc0[3 * dy + 1] = fmaf(t0, p1[dy], acc0[3 * dy + 1]);
+                acc1[3 * dy + 1] = fmaf(t1, p1[dy], acc1[3 * dy + 1]);
+                acc0[3 * dy + 2] = fmaf(t0, p2[dy], acc0[3 * dy + 2]);
+                acc1[3 * dy + 2] = fmaf(t1, p2[dy], acc1[3 * dy + 2]);
             }
-            for (int i = tid; i < kWChunk * 4; i += 320) {
-                const int q = i & 3, px = i >> 2, xx = x0 + px;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (xx < w) v = __ldg(reinterpret_cast<const uint4 *>(act + (((size_t)img * h + y) * w + xx) * kC + q * 8));
-                *reinterpret_cast<uint4 *>(sT + px * kC + q * 8) = v;
+            // bias: the sum of dZ (the tensor, or the plane's centre)
+            b0 += first_layer ? t0 : (x < w ? p1[1] : 0.f);
+            b1 += t1;
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                p0[dy] = p1[dy];
+                p1[dy] = p2[dy];
             }
-        } else {
-            // plane = dZ of the last layer (this row); act = its input (3 rows)
-            for (int i = tid; i < kWChunk; i += 320) {
-                const int xx = x0 + i;
-                sG[i] = xx < w ? plane[((size_t)img * h + y) * w + xx] : 0.f;
-            }
-            for (int i = tid; i < 3 * (kWChunk + 2) * 4; i += 320) {
-                const int q = i & 3, px = (i >> 2) % (kWChunk + 2), dy = (i >> 2) / (kWChunk + 2);
-                const int yy = y + dy - 1, xx = x0 - 1 + px;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (yy >= 0 && yy < h && xx >= 0 && xx < w)
-                    v = __ldg(reinterpret_cast<const uint4 *>(act + (((size_t)img * h + yy) * w + xx) * kC + q * 8));
-                *reinterpret_cast<uint4 *>(sT + (dy * (kWChunk + 2) + px) * kC + q * 8) = v;
-            }
-        }
-        __syncthreads();
-        if (j <= 9) {
-            const int tap = j < 9 ? j : 0, dy = tap / 3, dx = tap % 3;
-            if (first_layer) {
-                for (int k = 0; k < kWChunk; ++k) {
-                    const float g = __bfloat162float(sT[k * kC + c]);
-                    acc = fmaf(g, j < 9 ? sP[dy * (kWChunk + 2) + k + dx] : 1.f, acc);
-                }
-            } else {
-                for (int k = 0; k < kWChunk; ++k) {
-                    const float a = j < 9 ? __bfloat162float(sT[(dy * (kWChunk + 2) + k + dx) * kC + c]) : 1.f;
-                    acc = fmaf(sG[k], a, acc);
-                }
-            }
-        }
-    }
-    if (j < 9) {
-        // first layer: dW0[c][0][j]; last layer: dW4[0][c][j]
-        atomicAdd(dW + c * 9 + j, acc);
-    } else if (j == 9) {
-        if (first_layer) atomicAdd(db + c, acc);
-        else if (c == 0) {
-            // bias of the last layer: every c accumulated the same sum; use c = 0
-            atomicAdd(db, acc);
         }
     }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int tap = first_layer ? k : 8 - k;
+        const float s0 = acc0[k] + __shfl_xor_sync(0xffffffffu, acc0[k], 16);
+        const float s1 = acc1[k] + __shfl_xor_sync(0xffffffffu, acc1[k], 16);
+        atomicAdd(&sum[(c + half) * 9 + tap], half ? s1 : s0);
+    }
+    b0 += __shfl_xor_sync(0xffffffffu, b0, 16);
+    b1 += __shfl_xor_sync(0xffffffffu, b1, 16);
+    atomicAdd(&sum[kC * 9 + c + half], half ? b1 : b0);
+    __syncthreads();
+    for (int i = tid; i < kC * 9; i += 32 * kEWarps) atomicAdd(dW + i, sum[i]);   // dW0[co][0][tap], dW4[0][ci][tap]
+    if (tid < (first_layer ? kC : 1)) atomicAdd(db + tid, sum[kC * 9 + tid]);
 }
 
 // bf16 B operands from the fp32 master parameters (one thread per element).
@@ -659,17 +683,17 @@ cudaError_t launch_wgrad_mid(const bf16 *act, const bf16 *dz, int n, int h, int 
                              cudaStream_t cs) {
     cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_wgrad_mid), kWSmem);
     if (e != cudaSuccess) return e;
-    const int total = n * h * ((w + kWChunk - 1) / kWChunk);
-    const int grid = std::max(1, std::min(total, 3 * sm_count()));
-    k_wgrad_mid<<<grid, 128, kWSmem, cs>>>(act, dz, n, h, w, dW, db, err);
+    const int total = n * ((h + kWRowsT - 1) / kWRowsT) * ((w + kTilePx - 1) / kTilePx);
+    const int grid = std::max(1, std::min(total, 2 * sm_count()));
+    k_wgrad_mid<<<grid, kWThreads, kWSmem, cs>>>(act, dz, n, h, w, dW, db, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_wgrad_edge(const float *plane, const bf16 *act, int first, int n, int h, int w, float *dW,
                               float *db, cudaStream_t cs) {
-    const int total = n * h * ((w + kWChunk - 1) / kWChunk);
-    const int grid = std::max(1, std::min(total, 2 * sm_count()));
-    k_wgrad_edge<<<grid, 320, 0, cs>>>(plane, act, first, n, h, w, dW, db);
+    const int total = n * h * ((w + 2 * kERun - 1) / (2 * kERun));
+    const int grid = std::max(1, std::min((total + kEWarps - 1) / kEWarps, 2 * sm_count()));
+    k_wgrad_edge<<<grid, 32 * kEWarps, 0, cs>>>(plane, act, first, n, h, w, dW, db);
     return cudaGetLastError();
 }
 

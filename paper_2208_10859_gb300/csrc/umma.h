@@ -38,6 +38,12 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// "MN-major" operands: rows (M or N) contiguous instead of K.  The core
+// matrix is 8 K x 8 rows, 16 bytes (8 rows) per K; LBO is then the distance
+// between core matrices adjacent along K, SBO between those adjacent along
+// the rows.
+constexpr uint32_t kAMnMajor = 1u << 15, kBMnMajor = 1u << 16;
+
 // Warp-wide TMEM allocation of `cols` columns (a power of two >= 32); the
 // TMEM address is written to *dst (shared memory).
 template <int COLS>
