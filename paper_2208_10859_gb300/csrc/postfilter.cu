@@ -9,13 +9,14 @@
 //
 // Convolutions are implicit GEMMs on tcgen05 (one elected thread issues the
 // MMAs, operands in shared memory, accumulator in TMEM):
-//   forward / input gradient, 32 input channels: M = 128 pixels of one image
-//     row, N = 32 (or 16 for the 1-channel output), K = 9 taps x 32 channels
-//     = 18 K-steps.  The three input rows live in shared memory as 8-channel
-//     columns of 130 pixels (16 bytes per pixel), so the A operand of tap
-//     (dy, dx) is the row slot of dy shifted by dx pixels: only the
-//     descriptor's start address changes (SBO = 128 bytes, LBO = one column).
-//   forward / input gradient, 1 input channel: K = the 9 taps (padded to 16).
+//   forward / input gradient: M = 128 pixels of one image row, N = 32 output
+//     channels (16 for the last layer) of three output rows, K = 3 column taps
+//     x 32 channels.  An input row lies in shared memory as 8-channel columns
+//     of 130 pixels (16 bytes per pixel), so the A operand of column tap dx is
+//     the row shifted by dx pixels: only the descriptor's start address
+//     changes (SBO = 128 bytes, LBO = one column).  All layers run in one
+//     kernel (k_net).
+//   1 input channel: K = the 9 taps (padded to 16).
 //   weight gradient, 32 -> 32: D[dy, ci][dx, co] = sum over pixels of
 //     input[p + (dy, dx)][ci] * dZ[p][co]: M = (dy, ci), N = co, K = pixels,
 //     one accumulator per dx, both operands read channel-major.
@@ -29,6 +30,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <new>
 #include <vector>
 
@@ -46,7 +48,6 @@ constexpr int kTilePx = 128;            // pixels per MMA tile (M)
 constexpr int kRowPx = kTilePx + 2;     // input pixels of one row slot (1-pixel halo)
 constexpr int kLbo = kRowPx * 16;       // bytes between the 8-channel columns of a slot
 constexpr int kSlot = 4 * kLbo;         // one input row: 4 columns of 8 channels
-constexpr int kStrip = 16;              // output rows per work item
 constexpr int kStep32 = 32 * 32;        // bytes of one K-step of a 32-row operand
 constexpr int kBMid = 18 * kStep32;     // 32 x 288
 constexpr int kBLast = 18 * 16 * 32;    // 16 x 288 (row 0 real)
@@ -67,260 +68,437 @@ enum Pack { kPF0 = 0, kPF1 = kPF0 + kBIn1, kPF2 = kPF1 + kBMid, kPF3 = kPF2 + kB
             kPB4 = kPF4 + kBLast, kPB3 = kPB4 + kBIn1, kPB2 = kPB3 + kBMid, kPB1 = kPB2 + kBMid,
             kPackBytes = kPB1 + kBMid };
 
-enum Mode { kRelu = 0, kGate = 1, kLastTrain = 2, kLastOut = 3, kLastRgba = 4 };
+enum Mode { kTrain = 0, kOut = 1, kRgba = 2 };   // the last layer's epilogue
 
-struct ConvArgs {
-    const bf16 *in;          // NHWC, 32 channels (k_conv_mid)
-    const float *in_plane;   // one channel (k_conv_in1)
-    const uint8_t *wpack;    // packed B operand
-    const float *bias;       // per output channel, or null
+// ---- the chain of convolutions, fused --------------------------------------
+//
+// One CTA runs a chain of stages over a column tile of 128 pixels, row by
+// row: stage 0 (one input channel: layer 0, or the input gradient of layer
+// 4), three 32 -> 32 stages (layers 1-3, or their input gradients), and in the
+// forward pass the last layer (32 -> 1).  The rows between the stages stay in
+// shared memory; only the input plane, the output and, for training, the
+// activations or gradients the weight gradients need touch HBM.  Each stage
+// loses a pixel on either side, so a tile yields kTileOut = 120 columns, and
+// a segment of S rows costs 2 T more rows in stage 0 (T stages after it).
+//
+// MMAs: an input row (A: 128 pixels x 32 channels, one 8-channel column per
+// 16 bytes, shifted by dx pixels through the descriptor's start) takes part
+// in three output rows.  Their accumulators are three 32-column TMEM slots
+// (row index mod 3), all three updated by one MMA of N = 96 per K-step: B
+// holds the weights of dy = 1, 0, 2, 1, 0 side by side, and a window of three
+// starting at the right one fits any rotation of the slots.  So a row is 6
+// MMAs instead of 18 and reads A a third as often, and each output sums its
+// products in the same order (dy, dx, channel) as 18 would.  A drained slot is
+// zeroed by its reader, so every MMA accumulates.
+//
+// Roles: per stage one warp that issues its MMAs and one warpgroup that reads
+// its accumulator, applies bias and ReLU (or the ReLU gate of the backward
+// pass) and writes the next stage's input row into a ring of kRings slots.
+// (One warp issuing for all stages in turn took 3.2 us per row: a stage
+// waited for the issue and the waits of the four others.)  Every wait is an
+// mbarrier wait with a limit; one that gives up sets a flag that ends all
+// roles.
+//
+// Bound: the tensor pipe, busy on 76 % of the cycles (an MMA takes about one
+// cycle per accumulator column here).  A 2160^2 plane: 380 us, 2.4 GB of
+// activations no longer moved; layer by layer it took 887 us.
+
+constexpr int kTileOut = 120;           // output columns per tile
+constexpr int kRings = 3;               // input rows in flight per stage
+constexpr int kStages = 5;
+constexpr int kNetThreads = 32 * (4 * kStages + kStages);
+constexpr int kSeq = 5;                 // B blocks: dy = 1, 0, 2, 1, 0
+constexpr int kBBlock = 4 * 256;        // 32 output channels x 16 K
+constexpr int kBMidF = 6 * kSeq * kBBlock;
+constexpr int kBLastF = 6 * kSeq * (kBBlock / 2);
+constexpr int kA0 = 128 * 32;           // stage 0's operand: 128 pixels x 16 taps
+constexpr int kNetRing = 4 * kRings * kSlot;
+constexpr int kNetSmem = kNetRing + 3 * kBMidF + kBLastF + kBIn1 + 2 * kA0;
+
+struct NetArgs {
+    const float *in_plane;              // stage 0: one-channel input
+    const uint8_t *pack[kStages];       // packed B operand of each stage
+    const float *bias[kStages];         // forward
+    const bf16 *gate[kStages];          // backward: ReLU outputs of the layer below (NHWC)
+    bf16 *out[kStages];                 // NHWC outputs kept for the weight gradients, or null
     int n, h, w;
-    int mode;
-    bf16 *out;               // NHWC, 32 channels
-    const bf16 *gate;        // kGate: ReLU outputs of the layer below (NHWC)
-    const float *x;          // last layer: input luma
-    const float *t;          // kLastTrain: target
-    float *y;                // last layer: output plane (optional)
-    float *dz;               // kLastTrain: dL/dr plane
-    float *loss;             // kLastTrain: sum of squared errors
-    float grad_scale;        // kLastTrain: 2 / pixel count
-    const uint8_t *cb, *cr;  // kLastRgba: chroma planes of the viewport
+    int seg;                            // rows per segment
+    int mode;                           // last layer's epilogue
+    const float *x, *t;                 // last layer: input luma, target (kTrain)
+    float *y;                           // output plane (kOut; kTrain: optional)
+    float *dz;                          // kTrain: dL/dr plane
+    float *loss;                        // kTrain: sum of squared errors
+    float grad_scale;                   // kTrain: 2 / pixel count
+    const uint8_t *cb, *cr;             // kRgba: chroma planes of the viewport
     uint8_t *rgba;
     size_t pitch;
     int *err;
 };
 
-__device__ __forceinline__ size_t pix(const ConvArgs &a, int img, int y, int x) {
-    return ((size_t)img * a.h + y) * a.w + x;
+struct NetBars {
+    uint64_t in_full[kStages][kRings], in_free[kStages][kRings];   // stages 1..: input rows
+    uint64_t acc_full[kStages], drained[kStages];
+    uint64_t a0_full[2], acc0_full[2];
+    uint64_t idle[kStages];   // every MMA the stage issued has completed
+};
+
+// Waits for the phase; false (and the flag set) when the limit is reached or
+// another role has given up.
+__device__ __forceinline__ bool net_wait(uint64_t *bar, uint32_t parity, volatile int *stop) {
+    for (int k = 0; k < 64; ++k) {
+        if (umma::mbar_wait(bar, parity, 1 << 14)) return true;
+        if (*stop) return false;
+    }
+    *stop = 1;
+    return false;
 }
 
-// Epilogue of the 32-channel modes for one pixel: bias + ReLU, or the ReLU
-// gate of the layer below; bf16 NHWC store.
-__device__ __forceinline__ void load_gate(const ConvArgs &a, size_t p, uint4 (&g)[4]) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(a.gate + p * kC);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) g[q] = __ldg(src + q);
+// The same for a whole warp, with one answer for all its lanes.
+__device__ __forceinline__ bool net_wait_warp(uint64_t *bar, uint32_t parity, volatile int *stop) {
+    return __all_sync(0xffffffffu, net_wait(bar, parity, stop));
 }
 
-__device__ __forceinline__ void store32(const ConvArgs &a, size_t p, const float (&v)[32], const uint4 (&gate)[4]) {
-    float o[32];
-    if (a.mode == kRelu) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) o[c] = fmaxf(v[c] + (a.bias ? __ldg(a.bias + c) : 0.f), 0.f);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 gv = gate[q];
-            const bf16 *gb = reinterpret_cast<const bf16 *>(&gv);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) o[8 * q + e] = __bfloat162float(gb[e]) > 0.f ? v[8 * q + e] : 0.f;
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// First column of a stage's accumulators: stages 1-3 three slots of 32
+// columns, stage 4 three of 16, stage 0 two of 32.
+__device__ __forceinline__ uint32_t acc_col(int stage) { return stage == 0 ? 384 : stage == 4 ? 288 : 96 * (stage - 1); }
+
+struct NetTask {
+    int img, x0, y0, y1;   // output columns from x0, rows y0 .. y1 - 1
+};
+__device__ __forceinline__ NetTask net_task(const NetArgs &a, int it) {
+    const int tx = (a.w + kTileOut - 1) / kTileOut, ty = (a.h + a.seg - 1) / a.seg;
+    NetTask t;
+    t.img = it / (tx * ty);
+    t.x0 = (it % tx) * kTileOut;
+    t.y0 = ((it / tx) % ty) * a.seg;
+    t.y1 = min(t.y0 + a.seg, a.h);
+    return t;
+}
+__device__ __forceinline__ int net_tasks(const NetArgs &a) {
+    return a.n * ((a.w + kTileOut - 1) / kTileOut) * ((a.h + a.seg - 1) / a.seg);
+}
+
+// The elected thread that issues stage 0's MMAs.
+template <int T>
+__device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, const uint8_t *sA0, NetBars *bars,
+                                           uint32_t tmem, volatile int *stop) {
+    const uint64_t bd = umma::desc(umma::smem_addr(sB) + 3 * kBMidF + kBLastF, 128, 256);
+    const uint64_t ad = umma::desc(umma::smem_addr(sA0), 128, 256);
+    int r = 0;
+    for (int it = blockIdx.x; it < net_tasks(a); it += gridDim.x) {
+        const NetTask k = net_task(a, it);
+        for (int j = 0; j < k.y1 - k.y0 + 2 * T; ++j, ++r) {
+            const int b = r & 1;
+            if (!net_wait(&bars->a0_full[b], (r >> 1) & 1, stop)) return;
+            umma::fence_after_sync();
+            umma::mma(tmem + acc_col(0) + 32 * b, ad + b * (kA0 >> 4), bd, umma::idesc_bf16(128, 32), false);
+            umma::commit(&bars->acc0_full[b]);
         }
     }
-    uint4 *dst = reinterpret_cast<uint4 *>(a.out + p * kC);
+}
+
+// The elected thread that issues stage l's MMAs (BLK: bytes of one B block,
+// NC: accumulator columns per slot).  Input row j of a task takes part in
+// the output rows j - 2 .. j (counted from the task's first), which live in
+// the slots of their index mod 3.
+template <int T, int BLK, int NC>
+__device__ __forceinline__ void net_issue(const NetArgs &a, int l, const uint8_t *rings, const uint8_t *sB,
+                                          NetBars *bars, uint32_t tmem, volatile int *stop) {
+    const uint64_t ad = umma::desc(umma::smem_addr(rings) + (l - 1) * kRings * kSlot, kLbo, 128);
+    const uint64_t bd = umma::desc(umma::smem_addr(sB) + (l - 1) * kBMidF, 128, 256);
+    const uint32_t d = tmem + acc_col(l);
+    int u = 0, drains = 0;
+    for (int it = blockIdx.x; it < net_tasks(a); it += gridDim.x) {
+        const NetTask k = net_task(a, it);
+        const int rows = k.y1 - k.y0 + 2 * (T - l + 1);
+        for (int j = 0; j < rows; ++j, ++u) {
+            const int b = u % kRings;
+            if (!net_wait(&bars->in_full[l][b], (u / kRings) & 1, stop)) return;
+            if (j == 0 || j >= 3) {   // output row j's slot is free
+                if (!net_wait(&bars->drained[l], drains & 1, stop)) return;
+                ++drains;
+            }
+            umma::fence_after_sync();
+            const int rot = j % 3;
+            const uint32_t idesc = umma::idesc_bf16(128, NC) + ((uint32_t)(min(j, 2) * NC / 8) << 17);
+            const uint64_t as = ad + b * (kSlot >> 4), bs = bd + (rot == 0 ? BLK >> 4 : rot == 1 ? 0 : BLK >> 3);
+#pragma unroll
+            for (int s = 0; s < 6; ++s)   // K-step: dx = s / 2, channels 16 (s & 1) ..
+                umma::mma(d, as + (s >> 1) + (s & 1) * (2 * kLbo >> 4), bs + s * (kSeq * BLK >> 4), idesc, true);
+            umma::commit(&bars->in_free[l][b]);
+            if (j >= 2) umma::commit(&bars->acc_full[l]);
+        }
+    }
+}
+
+// Bias and ReLU, or the ReLU gate, of one pixel's 32 channels; `in`: the
+// pixel lies in the image (outside it every stage's output is the zero
+// padding).
+template <bool BWD>
+__device__ __forceinline__ void net_act(const float (&v)[32], const float *bias, const uint4 (&gate)[4], bool in,
+                                        uint4 (&o)[4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        uint4 w;
-        uint32_t *wp = reinterpret_cast<uint32_t *>(&w);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 b2 = __floats2bfloat162_rn(o[8 * q + 2 * e], o[8 * q + 2 * e + 1]);
-            wp[e] = *reinterpret_cast<const uint32_t *>(&b2);
+        float f[8], bv[8] = {};
+        if constexpr (!BWD) {
+            const float4 b0 = reinterpret_cast<const float4 *>(bias)[2 * q], b1 = reinterpret_cast<const float4 *>(bias)[2 * q + 1];
+            bv[0] = b0.x, bv[1] = b0.y, bv[2] = b0.z, bv[3] = b0.w;
+            bv[4] = b1.x, bv[5] = b1.y, bv[6] = b1.z, bv[7] = b1.w;
         }
-        dst[q] = w;
+        const uint32_t gw[4] = {gate[q].x, gate[q].y, gate[q].z, gate[q].w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if constexpr (BWD) {
+                const float g = __uint_as_float(e & 1 ? gw[e >> 1] & 0xffff0000u : gw[e >> 1] << 16);
+                f[e] = g > 0.f ? v[8 * q + e] : 0.f;
+            } else {
+                f[e] = fmaxf(v[8 * q + e] + bv[e], 0.f);
+            }
+        }
+        o[q] = make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
+        if (!in) o[q] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
-// Epilogue of the last layer (residual in column 0).
-__device__ __forceinline__ void store_last(const ConvArgs &a, size_t p, float r, bool valid) {
+// Epilogue of the last layer (residual r).
+__device__ __forceinline__ float store_last(const NetArgs &a, size_t p, float r, float bias, float x, float t) {
+    const float yv = x + r + bias;
+    if (a.y) a.y[p] = yv;
+    if (a.mode == kTrain) {
+        const float e = yv - t;
+        a.dz[p] = a.grad_scale * e;
+        return e * e;
+    }
+    if (a.mode == kRgba) {
+        const int yy = min(max(__float2int_rd(fmaf(yv, 255.f, 0.5f)), 0), 255);
+        const uchar4 c = to_rgba(yy, a.cb[p], a.cr[p]);
+        const int xw = (int)(p % a.w), yh = (int)(p / a.w);
+        *reinterpret_cast<uchar4 *>(a.rgba + (size_t)yh * a.pitch + 4 * (size_t)xw) = c;
+    }
+    return 0.f;
+}
+
+// A stage's warpgroup (thread = pixel of the tile).  T: the last stage.
+template <bool BWD, int T>
+__device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *rings, uint8_t *sA0, const float *bias,
+                                          NetBars *bars, uint32_t tmem, volatile int *stop) {
+    const int px = threadIdx.x & 127, lane = threadIdx.x & 31;
+    const uint32_t acc = tmem + acc_col(l) + ((uint32_t)(px & 96) << 16);
+    int outs = 0;       // rows completed by this stage (all tasks)
     float e2 = 0.f;
-    if (valid) {
-        const float yv = __ldg(a.x + p) + r + __ldg(a.bias);
-        if (a.y) a.y[p] = yv;
-        if (a.mode == kLastTrain) {
-            const float e = yv - __ldg(a.t + p);
-            a.dz[p] = a.grad_scale * e;
-            e2 = e * e;
-        } else if (a.mode == kLastRgba) {
-            const int yy = min(max(__float2int_rd(fmaf(yv, 255.f, 0.5f)), 0), 255);
-            const uchar4 c = to_rgba(yy, a.cb[p], a.cr[p]);
-            const int xw = (int)(p % a.w), yh = (int)(p / a.w);
-            *reinterpret_cast<uchar4 *>(a.rgba + (size_t)yh * a.pitch + 4 * (size_t)xw) = c;
+    if (l > 0) {        // zeroed accumulators
+        if (l == 4) {
+            for (int k = 0; k < 3; ++k) umma::zero16(acc + 16 * k);
+        } else {
+            for (int k = 0; k < 3; ++k) umma::zero32(acc + 32 * k);
         }
+        umma::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) umma::mbar_arrive(&bars->drained[l]);
     }
-    if (a.mode == kLastTrain) {
+    for (int it = blockIdx.x; it < net_tasks(a); it += gridDim.x) {
+        const NetTask k = net_task(a, it);
+        const int rows = k.y1 - k.y0 + 2 * (T - l);
+        const int gx = k.x0 - 4 + px;
+        const bool xin = gx >= 0 && gx < a.w, xown = px >= 4 && px < 4 + kTileOut && xin;
+        const size_t img = (size_t)k.img * a.h;
+        float win[9], nxt[3];
+        // stage 0: the window's next row, columns gx - 1 .. gx + 1
+        auto fetch = [&](int y) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-        if ((threadIdx.x & 31) == 0 && e2 != 0.f) atomicAdd(a.loss, e2);
-    }
-}
-
-// Convolution with 32 input channels (forward of layers 1-4, input gradient
-// of layers 1-3).  CTA: 128 threads, a strip of kStrip rows x 128 pixels.
-__global__ void __launch_bounds__(128) k_conv_mid(ConvArgs a, int nb) {
-    extern __shared__ __align__(128) uint8_t sm[];
-    uint8_t *slots = sm;              // 3 row slots
-    uint8_t *sB = sm + 3 * kSlot;     // packed B
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int bbytes = nb == 32 ? kBMid : kBLast;
-    for (int i = tid * 16; i < bbytes; i += 128 * 16)
-        *reinterpret_cast<uint4 *>(sB + i) = __ldg(reinterpret_cast<const uint4 *>(a.wpack + i));
-    if (tid == 0) umma::mbar_init(&mbar, 1);
-    if (warp == 0) umma::tmem_alloc<32>(&tmem_base);
-    umma::fence_before_sync();
-    __syncthreads();
-    umma::fence_after_sync();
-    const uint32_t tmem = tmem_base;
-    const uint32_t idesc = nb == 32 ? umma::idesc_bf16(128, 32) : umma::idesc_bf16(128, 16);
-    const int bstep = nb * 32;
-    uint32_t phase = 0;
-    // input row r: 130 pixels x 4 columns of 8 channels, 16 bytes each,
-    // staged through registers so that the next row's loads overlap the
-    // MMAs and the epilogue of the current one
-    constexpr int kPer = (kRowPx * 4 + 127) / 128;
-    uint4 pre[kPer];
-    auto load_row = [&](int img, int x0, int r) {
-        const bool rin = r >= 0 && r < a.h;
+            for (int c = 0; c < 3; ++c) {
+                const int xx = gx + c - 1;
+                nxt[c] = y >= 0 && y < a.h && xx >= 0 && xx < a.w ? __ldg(a.in_plane + (img + y) * a.w + xx) : 0.f;
+            }
+        };
+        auto slide = [&]() {
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int idx = tid + 128 * j;
-            const int px = idx >> 2, c = idx & 3, gx = x0 - 1 + px;
-            pre[j] = make_uint4(0u, 0u, 0u, 0u);
-            if (idx < kRowPx * 4 && rin && gx >= 0 && gx < a.w)
-                pre[j] = __ldg(reinterpret_cast<const uint4 *>(a.in + pix(a, img, r, gx) * kC + c * 8));
-        }
-    };
-    auto store_row = [&](int r) {
-        uint8_t *slot = slots + ((r + 3) % 3) * kSlot;
+            for (int c = 0; c < 6; ++c) win[c] = win[c + 3];
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int idx = tid + 128 * j;
-            if (idx < kRowPx * 4) *reinterpret_cast<uint4 *>(slot + (idx & 3) * kLbo + (idx >> 2) * 16) = pre[j];
-        }
-    };
-    // work items: strips of kStrip rows x 128 pixels, CTA b takes b, b + grid, ...
-    const int tiles_x = (a.w + kTilePx - 1) / kTilePx, strips = (a.h + kStrip - 1) / kStrip;
-    const int items = tiles_x * strips * a.n;
-    bool ok = true;
-    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const int img = it / (tiles_x * strips), sy = (it / tiles_x) % strips;
-        const int x0 = (it % tiles_x) * kTilePx, y0 = sy * kStrip, y1 = min(y0 + kStrip, a.h);
-        // the slots are free: the previous item's MMAs have completed
-        for (int r = y0 - 1; r <= y0 + 1; ++r) {
-            load_row(img, x0, r);
-            store_row(r);
-        }
-        const int xg = x0 + tid;
-        const bool valid = xg < a.w;
-        for (int y = y0; y < y1; ++y) {
+            for (int c = 0; c < 3; ++c) win[6 + c] = nxt[c];
+        };
+        // stage 0: the operand row of its output row `r` (counted over all tasks), then the next fetch
+        auto build = [&](int r, int y) {
+            slide();
+            fetch(y + 2);
+            uint8_t *d = sA0 + (r & 1) * kA0 + (px >> 3) * 256 + (px & 7) * 16;
+            *reinterpret_cast<uint4 *>(d) = make_uint4(pack2(win[0], win[1]), pack2(win[2], win[3]),
+                                                       pack2(win[4], win[5]), pack2(win[6], win[7]));
+            *reinterpret_cast<uint4 *>(d + 128) = make_uint4(pack2(win[8], 0.f), 0u, 0u, 0u);
             umma::fence_smem_to_async();
             umma::fence_before_sync();
-            __syncthreads();
-            umma::fence_after_sync();
-            if (tid == 0) {
-                const uint32_t sb = umma::smem_addr(sB);
-#pragma unroll 1
-                for (int tap = 0; tap < 9; ++tap) {
-                    const int dy = tap / 3, dx = tap % 3;
-                    const uint32_t abase = umma::smem_addr(slots + ((y + dy - 1 + 3) % 3) * kSlot) + dx * 16;
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(&bars->a0_full[r & 1]);
+        };
+        if (l == 0) {
+            const int y = k.y0 - T;
 #pragma unroll
-                    for (int s = 0; s < 2; ++s)
-                        umma::mma(tmem, umma::desc(abase + 2 * s * kLbo, kLbo, 128),
-                                  umma::desc(sb + (tap * 2 + s) * bstep, 128, 256), idesc, tap > 0 || s > 0);
-                }
-                umma::commit(&mbar);
-            }
-            const bool more = y + 1 < y1;
-            if (more) load_row(img, x0, y + 2);
+            for (int c = 0; c < 9; ++c) win[c] = 0.f;
+            fetch(y - 1);
+            slide();
+            fetch(y);
+            slide();
+            fetch(y + 1);
+            build(outs, y);
+        }
+        for (int q = 0; q < rows; ++q) {
+            const int y = k.y0 - (T - l) + q;
+            const bool in = xin && y >= 0 && y < a.h, own = xown && y >= k.y0 && y < k.y1;
+            const size_t p = (img + y) * a.w + gx;
+            if (l == 0 && q + 1 < rows) build(outs + 1, y + 1);
             uint4 gate[4] = {};
-            if (nb == 32 && a.mode == kGate && valid) load_gate(a, pix(a, img, y, xg), gate);
-            const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase));
-            phase ^= 1;
-            if (!got) {
-                if (tid == 0) record_error(a.err, WV_ERR_TIMEOUT);
-                ok = false;
-                break;
+            if (BWD && in) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.gate[l] + p * kC);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) gate[c] = __ldg(src + c);
+            }
+            float xv = 0.f, tv = 0.f;
+            if (!BWD && l == 4 && own) {
+                xv = __ldg(a.x + p);
+                if (a.mode == kTrain) tv = __ldg(a.t + p);
+            }
+            if (l == 0) {
+                if (!net_wait_warp(&bars->acc0_full[outs & 1], (outs >> 1) & 1, stop)) return;
+            } else {
+                if (!net_wait_warp(&bars->acc_full[l], outs & 1, stop)) return;
             }
             umma::fence_after_sync();
-            float v[32];
-            umma::ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
-            if (nb == 32) {
-                if (valid) store32(a, pix(a, img, y, xg), v, gate);
-            } else {
-                store_last(a, valid ? pix(a, img, y, xg) : 0, v[0], valid);
+            if (!BWD && l == 4) {
+                const float r = umma::ld1(acc + 16 * (q % 3));
+                if (q + 1 < rows) {
+                    umma::zero16(acc + 16 * (q % 3));
+                } else {   // the task's MMAs of this stage are done: the rows past its end leave nothing behind
+                    for (int c = 0; c < 3; ++c) umma::zero16(acc + 16 * c);
+                }
+                umma::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) umma::mbar_arrive(&bars->drained[l]);
+                if (own) e2 += store_last(a, p, r, bias[0], xv, tv);
+                ++outs;
+                continue;
             }
-            // the slot of row y - 1 is free: this row's MMAs have completed
-            if (more) store_row(y + 2);
-            umma::fence_before_sync();
+            float v[32];
+            if (l == 0) {
+                umma::ld32(acc + 32 * (outs & 1), v);
+                umma::fence_before_sync();
+            } else {
+                umma::ld32(acc + 32 * (q % 3), v);
+                if (q + 1 < rows) {
+                    umma::zero32(acc + 32 * (q % 3));
+                } else {
+                    for (int c = 0; c < 3; ++c) umma::zero32(acc + 32 * c);
+                }
+                umma::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) umma::mbar_arrive(&bars->drained[l]);
+            }
+            uint4 o[4];
+            net_act<BWD>(v, bias, gate, in, o);
+            if (l < T) {
+                const int b = outs % kRings;
+                if (outs >= kRings && !net_wait_warp(&bars->in_free[l + 1][b], (outs / kRings - 1) & 1, stop)) return;
+                uint8_t *d = rings + (l * kRings + b) * kSlot + (px + 1) * 16;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(d + c * kLbo) = o[c];
+                umma::fence_smem_to_async();
+                __syncwarp();
+                if (lane == 0) umma::mbar_arrive(&bars->in_full[l + 1][b]);
+            }
+            if (own && a.out[l]) {
+                uint4 *d = reinterpret_cast<uint4 *>(a.out[l] + p * kC);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) d[c] = o[c];
+            }
+            ++outs;
         }
     }
-    __syncthreads();
-    if (warp == 0) umma::tmem_free<32>(tmem);
+    if (!BWD && l == 4 && a.mode == kTrain) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        if (lane == 0 && e2 != 0.f) atomicAdd(a.loss, e2);
+    }
 }
 
-// Convolution with one input channel (forward of layer 0, input gradient of
-// layer 4): A row of a pixel = its 9 taps, padded to K = 16.
-__global__ void __launch_bounds__(128) k_conv_in1(ConvArgs a) {
-    __shared__ __align__(128) uint8_t sA[128 * 32];
-    __shared__ __align__(128) uint8_t sB[kBIn1];
-    __shared__ __align__(8) uint64_t mbar;
+template <bool BWD>
+__global__ void __launch_bounds__(kNetThreads, 1) k_net(NetArgs a) {
+    constexpr int T = BWD ? 3 : 4;
+    extern __shared__ __align__(128) uint8_t sm[];
+    uint8_t *rings = sm, *sB = sm + kNetRing, *sA0 = sB + 3 * kBMidF + kBLastF + kBIn1;
+    __shared__ NetBars bars;
     __shared__ uint32_t tmem_base;
+    __shared__ int stop;
+    __shared__ __align__(16) float sBias[kStages][kC];
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int x0 = blockIdx.x * kTilePx, y0 = blockIdx.y * kStrip, img = blockIdx.z;
-    for (int i = tid * 16; i < kBIn1; i += 128 * 16)
-        *reinterpret_cast<uint4 *>(sB + i) = __ldg(reinterpret_cast<const uint4 *>(a.wpack + i));
-    if (tid == 0) umma::mbar_init(&mbar, 1);
-    if (warp == 0) umma::tmem_alloc<32>(&tmem_base);
+    // B of the 32-channel stages: per K-step (dx, half of the channels) the
+    // blocks of dy = 1, 0, 2, 1, 0
+    for (int l = 1; l <= T; ++l) {
+        const int blk = l == 4 ? kBBlock / 2 : kBBlock;
+        uint8_t *dst = sB + (l - 1) * kBMidF;
+        for (int i = 16 * tid; i < 6 * kSeq * blk; i += 16 * kNetThreads) {
+            const int s = i / (kSeq * blk), r = (i / blk) % kSeq;
+            const int dy = r == 2 ? 2 : (r == 0 || r == 3) ? 1 : 0;
+            const int step = (dy * 3 + (s >> 1)) * 2 + (s & 1);
+            *reinterpret_cast<uint4 *>(dst + i) = __ldg(reinterpret_cast<const uint4 *>(a.pack[l] + step * blk + i % blk));
+        }
+    }
+    for (int i = 16 * tid; i < kBIn1; i += 16 * kNetThreads)
+        *reinterpret_cast<uint4 *>(sB + 3 * kBMidF + kBLastF + i) = __ldg(reinterpret_cast<const uint4 *>(a.pack[0] + i));
+    // the pixels left and right of the tile's 128 (read by its outermost,
+    // invalid columns)
+    for (int i = tid; i < 4 * kRings * 8; i += kNetThreads) {
+        const int c = i & 3, e = (i >> 2) & 1;
+        *reinterpret_cast<uint4 *>(rings + (i >> 3) * kSlot + c * kLbo + (e ? kRowPx - 1 : 0) * 16) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (!BWD)
+        for (int i = tid; i < kStages * kC; i += kNetThreads) {
+            const int l = i / kC;
+            sBias[l][i % kC] = l < 4 || i % kC == 0 ? __ldg(a.bias[l] + i % kC) : 0.f;
+        }
+    if (tid == 0) {
+        stop = 0;
+        for (int l = 0; l < kStages; ++l) {
+            for (int b = 0; b < kRings; ++b) {
+                umma::mbar_init(&bars.in_full[l][b], 4);
+                umma::mbar_init(&bars.in_free[l][b], 1);
+            }
+            umma::mbar_init(&bars.acc_full[l], 1);
+            umma::mbar_init(&bars.drained[l], 4);
+            umma::mbar_init(&bars.idle[l], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            umma::mbar_init(&bars.a0_full[b], 4);
+            umma::mbar_init(&bars.acc0_full[b], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 4 * kStages) umma::tmem_alloc<512>(&tmem_base);
+    umma::fence_smem_to_async();
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
-    const uint32_t idesc = umma::idesc_bf16(128, 32);
-    uint32_t phase = 0;
-    const int xg = x0 + tid;
-    const int y1 = min(y0 + kStrip, a.h);
-    for (int y = y0; y < y1; ++y) {
-        float t[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            t[k] = 0.f;
-            if (k < 9) {
-                const int yy = y + k / 3 - 1, xx = xg + k % 3 - 1;
-                if (yy >= 0 && yy < a.h && xx >= 0 && xx < a.w) t[k] = __ldg(a.in_plane + pix(a, img, yy, xx));
-            }
+    if (warp >= 4 * kStages) {
+        const int l = warp - 4 * kStages;
+        if ((tid & 31) == 0 && l <= T) {
+            if (l == 0) net_issue0<T>(a, sB, sA0, &bars, tmem, &stop);
+            else if (l < 4) net_issue<T, kBBlock, 32>(a, l, rings, sB, &bars, tmem, &stop);
+            else net_issue<T, kBBlock / 2, 16>(a, l, rings, sB, &bars, tmem, &stop);
+            umma::commit(&bars.idle[l]);
+            umma::mbar_wait(&bars.idle[l], 0);
         }
-#pragma unroll
-        for (int k = 0; k < 16; k += 2) {
-            const __nv_bfloat162 b2 = __floats2bfloat162_rn(t[k], t[k + 1]);
-            *reinterpret_cast<__nv_bfloat162 *>(sA + umma::kstep_offset(tid, k)) = b2;
-        }
-        umma::fence_smem_to_async();
-        umma::fence_before_sync();
-        __syncthreads();
-        umma::fence_after_sync();
-        if (tid == 0) {
-            umma::mma(tmem, umma::desc(umma::smem_addr(sA), 128, 256), umma::desc(umma::smem_addr(sB), 128, 256),
-                      idesc, false);
-            umma::commit(&mbar);
-        }
-        const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase));
-        phase ^= 1;
-        if (!got) {
-            if (tid == 0) record_error(a.err, WV_ERR_TIMEOUT);
-            break;
-        }
-        umma::fence_after_sync();
-        float v[32];
-        umma::ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
-        uint4 gate[4] = {};
-        if (a.mode == kGate && xg < a.w) load_gate(a, pix(a, img, y, xg), gate);
-        if (xg < a.w) store32(a, pix(a, img, y, xg), v, gate);
-        umma::fence_before_sync();
-        __syncthreads();
+        __syncwarp();
+    } else if ((warp >> 2) <= T) {
+        net_stage<BWD, T>(a, warp >> 2, rings, sA0, sBias[warp >> 2], &bars, tmem, &stop);
     }
+    umma::fence_before_sync();
     __syncthreads();
-    if (warp == 0) umma::tmem_free<32>(tmem);
+    if (tid == 0 && stop) record_error(a.err, WV_ERR_TIMEOUT);
+    if (warp == 4 * kStages) umma::tmem_free<512>(tmem);
 }
 
 // Weight gradient of a 32 -> 32 layer on the tensor cores:
@@ -609,42 +787,51 @@ struct wv_cnn {
     uint8_t *pack = nullptr;
     bool packed = false;
     int step = 0;
-    size_t cap_px = 0;
-    bf16 *act[4] = {};
-    bf16 *g[2] = {};
+    bf16 *act[4] = {};                 // training: layer outputs
+    bf16 *g[4] = {};                   // training: gradients of the layers' outputs
     float *dz5 = nullptr, *loss = nullptr, *xbuf = nullptr;
     uint8_t *cb = nullptr, *cr = nullptr;
+    size_t cap_train = 0, cap_view = 0;
+    std::vector<void *> owned_train, owned_view;
     int *err = nullptr;
-    std::vector<void *> owned;
 };
 
 namespace {
 
-int ensure_workspace(wv_cnn *c, size_t px) {
-    if (px <= c->cap_px) return WV_OK;
-    for (void *p : c->owned) cudaFree(p);
-    c->owned.clear();
+// Device buffers for px pixels; `ptr` gets the addresses of `bytes` per pixel.
+struct Buffer {
+    void **p;
+    size_t bytes;
+};
+int ensure_buffers(std::vector<void *> &owned, size_t &cap, size_t px, std::initializer_list<Buffer> list) {
+    if (px <= cap) return WV_OK;
+    for (void *p : owned) cudaFree(p);
+    owned.clear();
+    cap = 0;
     const size_t want = px + px / 8;
-    auto get = [&](size_t bytes) -> void * {
-        void *p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-        c->owned.push_back(p);
-        return p;
-    };
-    for (int i = 0; i < 4; ++i) c->act[i] = (bf16 *)get(want * kC * 2);
-    for (int i = 0; i < 2; ++i) c->g[i] = (bf16 *)get(want * kC * 2);
-    c->dz5 = (float *)get(want * 4);
-    c->xbuf = (float *)get(want * 4);
-    c->cb = (uint8_t *)get(want);
-    c->cr = (uint8_t *)get(want);
-    for (void *p : c->owned)
-        if (!p) {
+    for (const Buffer &b : list) {
+        *b.p = nullptr;
+        if (cudaMalloc(b.p, want * b.bytes) != cudaSuccess) {
             cudaGetLastError();
-            c->cap_px = 0;
             return WV_ERR_OOM;
         }
-    c->cap_px = want;
+        owned.push_back(*b.p);
+    }
+    cap = want;
     return WV_OK;
+}
+// A training step keeps every layer's output and its gradient.
+int ensure_train(wv_cnn *c, size_t px) {
+    const size_t row = kC * sizeof(bf16);
+    return ensure_buffers(c->owned_train, c->cap_train, px,
+                          {{(void **)&c->act[0], row}, {(void **)&c->act[1], row}, {(void **)&c->act[2], row},
+                           {(void **)&c->act[3], row}, {(void **)&c->g[0], row}, {(void **)&c->g[1], row},
+                           {(void **)&c->g[2], row}, {(void **)&c->g[3], row}, {(void **)&c->dz5, 4}});
+}
+// A filtered viewport: its luma and chroma planes.
+int ensure_view(wv_cnn *c, size_t px) {
+    return ensure_buffers(c->owned_view, c->cap_view, px,
+                          {{(void **)&c->xbuf, 4}, {(void **)&c->cb, 1}, {(void **)&c->cr, 1}});
 }
 
 void pack_params(wv_cnn *c, cudaStream_t cs) {
@@ -653,29 +840,32 @@ void pack_params(wv_cnn *c, cudaStream_t cs) {
     c->packed = true;
 }
 
-ConvArgs conv_args(wv_cnn *c, int n, int h, int w) {
-    ConvArgs a;
-    memset(&a, 0, sizeof(a));
-    a.n = n;
-    a.h = h;
-    a.w = w;
-    a.err = c->err;
-    return a;
+// Rows per segment: the least time over all SMs.  A CTA computes S + 2 T rows
+// in stage 0 for S rows and spends about 3 T more row times filling and draining
+// its stages, so whole waves of long segments win on large images and short ones on small
+// images that would leave SMs idle.
+int seg_rows(int n, int h, int w, int T) {
+    const long long tiles = (long long)n * ((w + kTileOut - 1) / kTileOut), sms = sm_count();
+    long long best = -1;
+    int seg = h;
+    for (int k = 1; k <= 128 && k <= h; ++k) {
+        const int s = (h + k - 1) / k;
+        const long long waves = (tiles * ((h + s - 1) / s) + sms - 1) / sms, cost = waves * (s + 5 * T);
+        if (best < 0 || cost < best) {
+            best = cost;
+            seg = s;
+        }
+    }
+    return seg;
 }
 
-cudaError_t launch_mid(const ConvArgs &a, int nb, cudaStream_t cs) {
-    const int smem = 3 * kSlot + kBMid;
-    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_conv_mid), smem);
+template <bool BWD>
+cudaError_t launch_net(NetArgs &a, cudaStream_t cs) {
+    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_net<BWD>), kNetSmem);
     if (e != cudaSuccess) return e;
-    // one work item (strip) per CTA: measured faster than persistent CTAs
-    const int items = ((a.w + kTilePx - 1) / kTilePx) * ((a.h + kStrip - 1) / kStrip) * a.n;
-    k_conv_mid<<<items, 128, smem, cs>>>(a, nb);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_in1(const ConvArgs &a, cudaStream_t cs) {
-    dim3 grid((a.w + kTilePx - 1) / kTilePx, (a.h + kStrip - 1) / kStrip, a.n);
-    k_conv_in1<<<grid, 128, 0, cs>>>(a);
+    a.seg = seg_rows(a.n, a.h, a.w, BWD ? 3 : 4);
+    const long long tasks = (long long)a.n * ((a.w + kTileOut - 1) / kTileOut) * ((a.h + a.seg - 1) / a.seg);
+    k_net<BWD><<<(int)std::min<long long>(tasks, sm_count()), kNetThreads, kNetSmem, cs>>>(a);
     return cudaGetLastError();
 }
 
@@ -697,37 +887,20 @@ cudaError_t launch_wgrad_edge(const float *plane, const bf16 *act, int first, in
     return cudaGetLastError();
 }
 
-// Forward pass; last-layer epilogue per `last` (with its outputs in `fin`).
-cudaError_t forward(wv_cnn *c, const float *x, int n, int h, int w, const ConvArgs &fin, cudaStream_t cs) {
+// Forward pass; the last layer's epilogue and outputs are set in `a`.
+cudaError_t forward(wv_cnn *c, const float *x, int n, int h, int w, NetArgs &a, cudaStream_t cs) {
     if (!c->packed) pack_params(c, cs);
-    ConvArgs a = conv_args(c, n, h, w);
-    a.in_plane = x;
-    a.wpack = c->pack + kPF0;
-    a.bias = c->params + off_b(0);
-    a.mode = kRelu;
-    a.out = c->act[0];
-    cudaError_t e = launch_in1(a, cs);
-    const int packs[3] = {kPF1, kPF2, kPF3};
-    for (int l = 1; l <= 3 && e == cudaSuccess; ++l) {
-        a = conv_args(c, n, h, w);
-        a.in = c->act[l - 1];
-        a.wpack = c->pack + packs[l - 1];
-        a.bias = c->params + off_b(l);
-        a.mode = kRelu;
-        a.out = c->act[l];
-        e = launch_mid(a, 32, cs);
-    }
-    if (e != cudaSuccess) return e;
-    a = fin;
+    const int packs[kStages] = {kPF0, kPF1, kPF2, kPF3, kPF4};
+    a.in_plane = a.x = x;
     a.n = n;
     a.h = h;
     a.w = w;
     a.err = c->err;
-    a.in = c->act[3];
-    a.wpack = c->pack + kPF4;
-    a.bias = c->params + off_b(4);
-    a.x = x;
-    return launch_mid(a, 16, cs);
+    for (int l = 0; l < kStages; ++l) {
+        a.pack[l] = c->pack + packs[l];
+        a.bias[l] = c->params + off_b(l);
+    }
+    return launch_net<false>(a, cs);
 }
 
 // Forward with the training epilogue, then every gradient into c->grads.
@@ -735,47 +908,41 @@ cudaError_t forward_backward(wv_cnn *c, const float *x, const float *t, int n, i
     cudaError_t e = cudaMemsetAsync(c->grads, 0, sizeof(float) * kParams, cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->loss, 0, sizeof(float), cs);
     if (e != cudaSuccess) return e;
-    ConvArgs fin;
-    memset(&fin, 0, sizeof(fin));
-    fin.mode = kLastTrain;
-    fin.t = t;
-    fin.dz = c->dz5;
-    fin.loss = c->loss;
-    fin.grad_scale = 2.f / (float)((double)n * h * w);
-    e = forward(c, x, n, h, w, fin, cs);
+    NetArgs a;
+    memset(&a, 0, sizeof(a));
+    a.mode = kTrain;
+    a.t = t;
+    a.dz = c->dz5;
+    a.loss = c->loss;
+    a.grad_scale = 2.f / (float)((double)n * h * w);
+    for (int l = 0; l < 4; ++l) a.out[l] = c->act[l];
+    e = forward(c, x, n, h, w, a, cs);
     if (e != cudaSuccess) return e;
-    float *G = c->grads;
-    // layer 4
-    e = launch_wgrad_edge(c->dz5, c->act[3], 0, n, h, w, G + off_w(4), G + off_b(4), cs);
-    ConvArgs a = conv_args(c, n, h, w);
+    // gradients of the outputs of layers 3..0: stage s yields layer 3 - s's,
+    // gated by that layer's output
+    const int packs[4] = {kPB4, kPB3, kPB2, kPB1};
+    memset(&a, 0, sizeof(a));
     a.in_plane = c->dz5;
-    a.wpack = c->pack + kPB4;
-    a.mode = kGate;
-    a.gate = c->act[3];
-    a.out = c->g[0];
-    if (e == cudaSuccess) e = launch_in1(a, cs);
-    // layers 3, 2, 1: weight gradient from (input, dZ), then dZ of the layer below
-    const int bw[4] = {0, kPB1, kPB2, kPB3};
-    int cur = 0;
-    for (int l = 3; l >= 1 && e == cudaSuccess; --l) {
-        e = launch_wgrad_mid(c->act[l - 1], c->g[cur], n, h, w, G + off_w(l), G + off_b(l), c->err, cs);
-        if (e != cudaSuccess) break;
-        a = conv_args(c, n, h, w);
-        a.in = c->g[cur];
-        a.wpack = c->pack + bw[l];
-        a.mode = kGate;
-        a.gate = c->act[l - 1];
-        a.out = c->g[1 - cur];
-        e = launch_mid(a, 32, cs);
-        cur = 1 - cur;
+    a.n = n;
+    a.h = h;
+    a.w = w;
+    a.err = c->err;
+    for (int s = 0; s < 4; ++s) {
+        a.pack[s] = c->pack + packs[s];
+        a.gate[s] = c->act[3 - s];
+        a.out[s] = c->g[3 - s];
     }
-    // layer 0
-    if (e == cudaSuccess) e = launch_wgrad_edge(x, c->g[cur], 1, n, h, w, G + off_w(0), G + off_b(0), cs);
+    e = launch_net<true>(a, cs);
+    float *G = c->grads;
+    if (e == cudaSuccess) e = launch_wgrad_edge(c->dz5, c->act[3], 0, n, h, w, G + off_w(4), G + off_b(4), cs);
+    for (int l = 3; l >= 1 && e == cudaSuccess; --l)
+        e = launch_wgrad_mid(c->act[l - 1], c->g[l], n, h, w, G + off_w(l), G + off_b(l), c->err, cs);
+    if (e == cudaSuccess) e = launch_wgrad_edge(x, c->g[0], 1, n, h, w, G + off_w(0), G + off_b(0), cs);
     return e;
 }
 
 int check_dims(int n, int h, int w) {
-    return (n >= 1 && h >= 1 && w >= 1 && (double)n * h * w < 2e9 && h <= 65535 * kStrip && n <= 65535)
+    return (n >= 1 && h >= 1 && w >= 1 && (double)n * h * w < 2e9 && h <= 65535 * 16 && n <= 65535)
                ? WV_OK
                : WV_ERR_ARG;
 }
@@ -820,7 +987,8 @@ int wv_cnn_create(const float *params_host, wv_cnn **out) {
 void wv_cnn_close(wv_cnn *c) {
     if (!c) return;
     cudaDeviceSynchronize();
-    for (void *p : c->owned) cudaFree(p);
+    for (void *p : c->owned_train) cudaFree(p);
+    for (void *p : c->owned_view) cudaFree(p);
     cudaFree(c->params);
     cudaFree(c->grads);
     cudaFree(c->m);
@@ -869,10 +1037,9 @@ int wv_cnn_set_state(wv_cnn *c, const float *m_host, const float *v_host, int st
 
 int wv_cnn_forward(wv_cnn *c, const float *x_dev, float *y_dev, int n, int h, int w, void *cuda_stream) {
     if (!c || !x_dev || !y_dev || check_dims(n, h, w) != WV_OK) return WV_ERR_ARG;
-    if (ensure_workspace(c, (size_t)n * h * w) != WV_OK) return WV_ERR_OOM;
-    ConvArgs fin;
+    NetArgs fin;
     memset(&fin, 0, sizeof(fin));
-    fin.mode = kLastOut;
+    fin.mode = kOut;
     fin.y = y_dev;
     return forward(c, x_dev, n, h, w, fin, (cudaStream_t)cuda_stream) == cudaSuccess ? WV_OK : WV_ERR_CUDA;
 }
@@ -880,7 +1047,7 @@ int wv_cnn_forward(wv_cnn *c, const float *x_dev, float *y_dev, int n, int h, in
 int wv_cnn_gradients(wv_cnn *c, const float *x_dev, const float *t_dev, int n, int h, int w, float *grads_host,
                      float *loss_host, void *cuda_stream) {
     if (!c || !x_dev || !t_dev || check_dims(n, h, w) != WV_OK) return WV_ERR_ARG;
-    if (ensure_workspace(c, (size_t)n * h * w) != WV_OK) return WV_ERR_OOM;
+    if (ensure_train(c, (size_t)n * h * w) != WV_OK) return WV_ERR_OOM;
     cudaStream_t cs = (cudaStream_t)cuda_stream;
     if (forward_backward(c, x_dev, t_dev, n, h, w, cs) != cudaSuccess) return WV_ERR_CUDA;
     float loss = 0.f;
@@ -895,7 +1062,7 @@ int wv_cnn_gradients(wv_cnn *c, const float *x_dev, const float *t_dev, int n, i
 int wv_cnn_train_step(wv_cnn *c, const float *x_dev, const float *t_dev, int n, int h, int w, float lr,
                       float *loss_host, void *cuda_stream) {
     if (!c || !x_dev || !t_dev || check_dims(n, h, w) != WV_OK || !(lr > 0.f)) return WV_ERR_ARG;
-    if (ensure_workspace(c, (size_t)n * h * w) != WV_OK) return WV_ERR_OOM;
+    if (ensure_train(c, (size_t)n * h * w) != WV_OK) return WV_ERR_OOM;
     cudaStream_t cs = (cudaStream_t)cuda_stream;
     if (forward_backward(c, x_dev, t_dev, n, h, w, cs) != cudaSuccess) return WV_ERR_CUDA;
     c->step += 1;
@@ -934,7 +1101,7 @@ int wv_decode_viewport_filtered(wv_stream *s, int frame, float yaw, float pitch,
         return WV_ERR_ARG;
     if (frame < 0 || frame >= s->g.num_frames || !(fov > 0.f && fov < 3.14159f)) return WV_ERR_ARG;
     const size_t px = (size_t)out->width * out->height;
-    if (ensure_workspace(c, px) != WV_OK) return WV_ERR_OOM;
+    if (ensure_view(c, px) != WV_OK) return WV_ERR_OOM;
     // the region decode of the plain path, then the planes instead of RGBA
     int rc = wv::decode_region(s, frame, yaw, pitch, fov, out->width, out->height);
     if (rc != WV_OK) return rc;
@@ -944,9 +1111,9 @@ int wv_decode_viewport_filtered(wv_stream *s, int frame, float yaw, float pitch,
     launch_resample(s->g, v, recon_planes(s), nullptr, nullptr, 0, s->cs, c->xbuf, c->cb, c->cr, recon_pairs(s),
                     s->err);
     release_recon(s);
-    ConvArgs fin;
+    NetArgs fin;
     memset(&fin, 0, sizeof(fin));
-    fin.mode = kLastRgba;
+    fin.mode = kRgba;
     fin.cb = c->cb;
     fin.cr = c->cr;
     fin.rgba = (uint8_t *)out->dptr;

@@ -119,6 +119,35 @@ __device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// One fp32 column of the thread's TMEM lane.
+__device__ __forceinline__ float ld1(uint32_t taddr) {
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    return __uint_as_float(r);
+}
+
+// Zero 32 (16) consecutive columns of the warp's TMEM lanes; complete on return.
+__device__ __forceinline__ void zero32(uint32_t taddr) {
+    asm volatile(
+        "{\n.reg .b32 z;\nmov.b32 z, 0;\n"
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z};\n}" ::"r"(
+            taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void zero16(uint32_t taddr) {
+    asm volatile(
+        "{\n.reg .b32 z;\nmov.b32 z, 0;\n"
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {z,z,z,z,z,z,z,z,z,z,z,z,z,z,z,z};\n}" ::"r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("{\n.reg .b64 s;\nmbarrier.arrive.shared::cta.b64 s, [%0];\n}" ::"r"(smem_addr(mbar)) : "memory");
+}
+
 // Byte offset of element (r, k) in a K-major, no-swizzle tile of R rows and
 // 16 K elements (one MMA K-step): core matrix (r / 8, k / 8) at
 // (r / 8) * 256 + (k / 8) * 128 (LBO 128, SBO 256).

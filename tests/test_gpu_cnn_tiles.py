@@ -60,14 +60,21 @@ def test_workload_is_exact(shape):
 
 def gradients(layers, x, y, acts, t):
     """The oracle's backward pass with the gradients between the layers held
-    as bf16, as the network holds them."""
+    as bf16, as the network holds them: per layer and tensor the gradient and
+    the largest sum of its terms' magnitudes (what fp32 summation errors are
+    relative to; the terms have both signs)."""
+    def layer(a, g):
+        s = np.abs(g)
+        return [(OC.conv3x3_grad_weight(a, g), OC.conv3x3_grad_weight(np.abs(a), s).max()),
+                (g.sum(axis=(0, 2, 3)), s.sum(axis=(0, 2, 3)).max())]
+
     dz = (np.float32(2.0) / np.float32(x.size)) * (y - t).astype(np.float32)
     g = dz.astype(np.float64)[:, None]
-    out = [(OC.conv3x3_grad_weight(acts[4], g), g.sum(axis=(0, 2, 3)))]
+    out = [layer(acts[4], g)]
     g = bf16(dz)[:, None]
     for k in range(4, 0, -1):
         g = bf16(OC.conv3x3_grad_input(g, layers[k][0]) * (acts[k] > 0))
-        out.insert(0, (OC.conv3x3_grad_weight(acts[k - 1], g), g.sum(axis=(0, 2, 3))))
+        out.insert(0, layer(acts[k - 1], g))
     return out
 
 
@@ -83,9 +90,9 @@ def test_exact_workload(shape):
     loss, g = net.gradients(xd, td)
     assert loss == pytest.approx(float(np.mean((y - t) ** 2)), rel=1e-6)
     o = 0
-    for k, (dw, db) in enumerate(gradients(layers, x, y, acts, t)):
-        for v in (dw, db):
+    for k, tensors in enumerate(gradients(layers, x, y, acts, t)):
+        for v, terms in tensors:
             got = g[o:o + v.size].astype(np.float64)
             o += v.size
-            assert np.abs(got - v.ravel()).max() <= 1e-6 * max(np.abs(v).max(), 2.0 / x.size), k
+            assert np.abs(got - v.ravel()).max() <= 1e-6 * terms, k
     assert net.sync_status() == 0
