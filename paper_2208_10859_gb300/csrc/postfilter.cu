@@ -99,14 +99,17 @@ enum Mode { kTrain = 0, kOut = 1, kRgba = 2 };   // the last layer's epilogue
 // mbarrier wait with a limit; one that gives up sets a flag that ends all
 // roles.
 //
-// Bound: the tensor pipe, busy on 76 % of the cycles (an MMA takes about one
-// cycle per accumulator column here).  A 2160^2 plane: 380 us, 2.4 GB of
-// activations no longer moved; layer by layer it took 887 us.
+// Bound: the tensor pipe (an MMA takes about one cycle per accumulator column
+// here, 290 us of a 2160^2 plane's 306).  Layer by layer, 2.4 GB of
+// activations through HBM, the plane took 887 us.  Training adds 512 bytes a
+// pixel of activations and gradients kept: 144 us forward and 155 us for the
+// input gradients of 16 x 256^2 pixels (270 and 230 layer by layer).
 
 constexpr int kTileOut = 120;           // output columns per tile
 constexpr int kRings = 3;               // input rows in flight per stage
 constexpr int kStages = 5;
-constexpr int kNetThreads = 32 * (4 * kStages + kStages);
+// threads of a chain of T + 1 stages: a warpgroup and an issuing warp each
+__host__ __device__ constexpr int net_threads(bool bwd) { return 32 * 5 * (bwd ? 4 : kStages); }
 constexpr int kSeq = 5;                 // B blocks: dy = 1, 0, 2, 1, 0
 constexpr int kBBlock = 4 * 256;        // 32 output channels x 16 K
 constexpr int kBMidF = 6 * kSeq * kBBlock;
@@ -183,7 +186,7 @@ __device__ __forceinline__ int net_tasks(const NetArgs &a) {
     return a.n * ((a.w + kTileOut - 1) / kTileOut) * ((a.h + a.seg - 1) / a.seg);
 }
 
-// The elected thread that issues stage 0's MMAs.
+// The warp that issues stage 0's MMAs (control flow and operands uniform).
 template <int T>
 __device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, const uint8_t *sA0, NetBars *bars,
                                            uint32_t tmem, volatile int *stop) {
@@ -194,15 +197,18 @@ __device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, 
         const NetTask k = net_task(a, it);
         for (int j = 0; j < k.y1 - k.y0 + 2 * T; ++j, ++r) {
             const int b = r & 1;
-            if (!net_wait(&bars->a0_full[b], (r >> 1) & 1, stop)) return;
+            if (!net_wait_warp(&bars->a0_full[b], (r >> 1) & 1, stop)) return;
             umma::fence_after_sync();
-            umma::mma(tmem + acc_col(0) + 32 * b, ad + b * (kA0 >> 4), bd, umma::idesc_bf16(128, 32), false);
-            umma::commit(&bars->acc0_full[b]);
+            if (umma::elect_one()) {
+                umma::mma(tmem + acc_col(0) + 32 * b, ad + b * (kA0 >> 4), bd, umma::idesc_bf16(128, 32), false);
+                umma::commit(&bars->acc0_full[b]);
+            }
+            __syncwarp();
         }
     }
 }
 
-// The elected thread that issues stage l's MMAs (BLK: bytes of one B block,
+// The warp that issues stage l's MMAs (BLK: bytes of one B block,
 // NC: accumulator columns per slot).  Input row j of a task takes part in
 // the output rows j - 2 .. j (counted from the task's first), which live in
 // the slots of their index mod 3.
@@ -218,20 +224,23 @@ __device__ __forceinline__ void net_issue(const NetArgs &a, int l, const uint8_t
         const int rows = k.y1 - k.y0 + 2 * (T - l + 1);
         for (int j = 0; j < rows; ++j, ++u) {
             const int b = u % kRings;
-            if (!net_wait(&bars->in_full[l][b], (u / kRings) & 1, stop)) return;
+            if (!net_wait_warp(&bars->in_full[l][b], (u / kRings) & 1, stop)) return;
             if (j == 0 || j >= 3) {   // output row j's slot is free
-                if (!net_wait(&bars->drained[l], drains & 1, stop)) return;
+                if (!net_wait_warp(&bars->drained[l], drains & 1, stop)) return;
                 ++drains;
             }
             umma::fence_after_sync();
             const int rot = j % 3;
             const uint32_t idesc = umma::idesc_bf16(128, NC) + ((uint32_t)(min(j, 2) * NC / 8) << 17);
             const uint64_t as = ad + b * (kSlot >> 4), bs = bd + (rot == 0 ? BLK >> 4 : rot == 1 ? 0 : BLK >> 3);
+            if (umma::elect_one()) {
 #pragma unroll
-            for (int s = 0; s < 6; ++s)   // K-step: dx = s / 2, channels 16 (s & 1) ..
-                umma::mma(d, as + (s >> 1) + (s & 1) * (2 * kLbo >> 4), bs + s * (kSeq * BLK >> 4), idesc, true);
-            umma::commit(&bars->in_free[l][b]);
-            if (j >= 2) umma::commit(&bars->acc_full[l]);
+                for (int s = 0; s < 6; ++s)   // K-step: dx = s / 2, channels 16 (s & 1) ..
+                    umma::mma(d, as + (s >> 1) + (s & 1) * (2 * kLbo >> 4), bs + s * (kSeq * BLK >> 4), idesc, true);
+                umma::commit(&bars->in_free[l][b]);
+                if (j >= 2) umma::commit(&bars->acc_full[l]);
+            }
+            __syncwarp();
         }
     }
 }
@@ -346,17 +355,20 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
             fetch(y + 1);
             build(outs, y);
         }
+        uint4 gate[4] = {};   // fetched a row ahead
+        auto load_gate = [&](int y) {
+            if (BWD && xin && y >= 0 && y < a.h) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.gate[l] + ((img + y) * a.w + gx) * kC);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) gate[c] = __ldg(src + c);
+            }
+        };
+        load_gate(k.y0 - (T - l));
         for (int q = 0; q < rows; ++q) {
             const int y = k.y0 - (T - l) + q;
             const bool in = xin && y >= 0 && y < a.h, own = xown && y >= k.y0 && y < k.y1;
             const size_t p = (img + y) * a.w + gx;
             if (l == 0 && q + 1 < rows) build(outs + 1, y + 1);
-            uint4 gate[4] = {};
-            if (BWD && in) {
-                const uint4 *src = reinterpret_cast<const uint4 *>(a.gate[l] + p * kC);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) gate[c] = __ldg(src + c);
-            }
             float xv = 0.f, tv = 0.f;
             if (!BWD && l == 4 && own) {
                 xv = __ldg(a.x + p);
@@ -399,20 +411,29 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
             }
             uint4 o[4];
             net_act<BWD>(v, bias, gate, in, o);
-            if (l < T) {
-                const int b = outs % kRings;
-                if (outs >= kRings && !net_wait_warp(&bars->in_free[l + 1][b], (outs / kRings - 1) & 1, stop)) return;
-                uint8_t *d = rings + (l * kRings + b) * kSlot + (px + 1) * 16;
+            if (q + 1 < rows) load_gate(y + 1);
+            // into the next stage's ring (the last stage's rows only pass
+            // through it on their way to memory)
+            const int b = outs % kRings;
+            if (l < T && outs >= kRings && !net_wait_warp(&bars->in_free[l + 1][b], (outs / kRings - 1) & 1, stop)) return;
+            uint8_t *row = rings + (l * kRings + b) * kSlot + 16;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(d + c * kLbo) = o[c];
+            for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(row + px * 16 + c * kLbo) = o[c];
+            if (l < T) {
                 umma::fence_smem_to_async();
                 __syncwarp();
                 if (lane == 0) umma::mbar_arrive(&bars->in_full[l + 1][b]);
             }
-            if (own && a.out[l]) {
-                uint4 *d = reinterpret_cast<uint4 *>(a.out[l] + p * kC);
+            if (a.out[l] && y >= k.y0 && y < k.y1) {
+                // whole 64-byte pixels by four lanes each: a warp writes 512 contiguous bytes
+                __syncwarp();
+                uint4 *dst = reinterpret_cast<uint4 *>(a.out[l] + ((img + y) * a.w + k.x0 - 4) * kC);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) d[c] = o[c];
+                for (int c = 0; c < 4; ++c) {
+                    const int i = 128 * (px >> 5) + 32 * c + lane, x = i >> 2;
+                    if (x >= 4 && x < 4 + kTileOut && k.x0 - 4 + x < a.w)
+                        dst[i] = *reinterpret_cast<const uint4 *>(row + x * 16 + (i & 3) * kLbo);
+                }
             }
             ++outs;
         }
@@ -425,15 +446,15 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
 }
 
 template <bool BWD>
-__global__ void __launch_bounds__(kNetThreads, 1) k_net(NetArgs a) {
-    constexpr int T = BWD ? 3 : 4;
+__global__ void __launch_bounds__(net_threads(BWD), 1) k_net(NetArgs a) {
+    constexpr int T = BWD ? 3 : 4, kNetThreads = net_threads(BWD);
     extern __shared__ __align__(128) uint8_t sm[];
     uint8_t *rings = sm, *sB = sm + kNetRing, *sA0 = sB + 3 * kBMidF + kBLastF + kBIn1;
     __shared__ NetBars bars;
     __shared__ uint32_t tmem_base;
     __shared__ int stop;
     __shared__ __align__(16) float sBias[kStages][kC];
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform
     // B of the 32-channel stages: per K-step (dx, half of the channels) the
     // blocks of dy = 1, 0, 2, 1, 0
     for (int l = 1; l <= T; ++l) {
@@ -476,29 +497,29 @@ __global__ void __launch_bounds__(kNetThreads, 1) k_net(NetArgs a) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4 * kStages) umma::tmem_alloc<512>(&tmem_base);
+    if (warp == 4 * (T + 1)) umma::tmem_alloc<512>(&tmem_base);
     umma::fence_smem_to_async();
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = tmem_base;
-    if (warp >= 4 * kStages) {
-        const int l = warp - 4 * kStages;
-        if ((tid & 31) == 0 && l <= T) {
-            if (l == 0) net_issue0<T>(a, sB, sA0, &bars, tmem, &stop);
-            else if (l < 4) net_issue<T, kBBlock, 32>(a, l, rings, sB, &bars, tmem, &stop);
-            else net_issue<T, kBBlock / 2, 16>(a, l, rings, sB, &bars, tmem, &stop);
+    if (warp >= 4 * (T + 1)) {
+        const int l = warp - 4 * (T + 1);
+        if (l == 0) net_issue0<T>(a, sB, sA0, &bars, tmem, &stop);
+        else if (l < 4) net_issue<T, kBBlock, 32>(a, l, rings, sB, &bars, tmem, &stop);
+        else net_issue<T, kBBlock / 2, 16>(a, l, rings, sB, &bars, tmem, &stop);
+        if (umma::elect_one()) {
             umma::commit(&bars.idle[l]);
             umma::mbar_wait(&bars.idle[l], 0);
         }
         __syncwarp();
-    } else if ((warp >> 2) <= T) {
+    } else {
         net_stage<BWD, T>(a, warp >> 2, rings, sA0, sBias[warp >> 2], &bars, tmem, &stop);
     }
     umma::fence_before_sync();
     __syncthreads();
     if (tid == 0 && stop) record_error(a.err, WV_ERR_TIMEOUT);
-    if (warp == 4 * kStages) umma::tmem_free<512>(tmem);
+    if (warp == 4 * (T + 1)) umma::tmem_free<512>(tmem);
 }
 
 // Weight gradient of a 32 -> 32 layer on the tensor cores:
@@ -517,8 +538,10 @@ __global__ void __launch_bounds__(kNetThreads, 1) k_net(NetArgs a) {
 //
 // Bound: the MMAs' reads of A (4 KB per 16 pixels and dx) and the 128 bytes
 // per pixel from HBM, about 20 us each for 16 x 256^2 pixels; two CTAs per SM
-// so that one's loads run under the other's MMAs.  Measured 79 us; the form
-// with both operands transposed through shared memory by the threads 434 us.
+// so that one's loads run under the other's MMAs (one CTA with two operand
+// buffers: 88 us, too few warps issuing loads).  Measured
+// 71 us; the form with both operands transposed through shared memory by the
+// threads took 434 us.
 constexpr int kWRowsT = 4;                              // dz rows per tile
 constexpr int kWThreads = 256;
 constexpr int kWAct = (kWRowsT + 3) * kSlot;            // kWRowsT + 2 rows, one more that the last M reads
@@ -535,12 +558,11 @@ __device__ __forceinline__ void cp_async16(uint8_t *dst, const void *src, bool f
 __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restrict__ act, const bf16 *__restrict__ dz,
                                                            int n, int h, int w, float *dW, float *db, int *err) {
     extern __shared__ __align__(128) uint8_t sm[];
-    uint8_t *sAct = sm, *sDz = sm + kWAct;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ float sBias[kC];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    if (tid == 0) umma::mbar_init(&mbar, 1);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform
+    if (tid == 0) umma::mbar_init(&mbar, 3);
     if (tid < kC) sBias[tid] = 0.f;
     if (warp == 0) umma::tmem_alloc<128>(&tmem_base);
     umma::fence_before_sync();
@@ -550,66 +572,81 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restri
     const uint32_t idesc = umma::idesc_bf16(128, 32) | umma::kAMnMajor | umma::kBMnMajor;
     const int tx = (w + kTilePx - 1) / kTilePx, ty = (h + kWRowsT - 1) / kWRowsT;
     const int total = n * tx * ty;
-    uint32_t phase = 0;
-    bool first = true, ok = true;
-    float bsum[8] = {};   // channels 8 (tid & 3) ..
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+    const int q = tid & 3, p0 = tid >> 2;   // this thread's 8 channels and first pixel of a row
+    uint8_t *buf = sm;
+    auto load = [&](int it) {
         const int x0 = (it % tx) * kTilePx, y0 = ((it / tx) % ty) * kWRowsT, img = it / (tx * ty);
-        const int rows = min(kWRowsT, h - y0);
-        const int steps = (min(kTilePx, w - x0) + 15) / 16;   // K-steps of 16 pixels
-        const int apx = 16 * steps + 2;
-        for (int i = tid; i < (rows + 2) * apx * 4; i += kWThreads) {
-            const int q = i & 3, px = (i >> 2) % apx, r = (i >> 2) / apx;
-            const int yy = y0 + r - 1, xx = x0 - 1 + px;
-            const bool in = yy >= 0 && yy < h && xx >= 0 && xx < w;
-            cp_async16(sAct + r * kSlot + q * kLbo + px * 16,
-                       in ? act + (((size_t)img * h + yy) * w + xx) * kC + q * 8 : act, in);
-        }
-        for (int i = tid; i < rows * steps * 64; i += kWThreads) {
-            const int q = i & 3, px = (i >> 2) % (16 * steps), r = (i >> 2) / (16 * steps);
-            const int yy = y0 + r, xx = x0 + px;
-            const bool in = xx < w;
-            cp_async16(sDz + r * kSlot + q * kLbo + px * 16,
-                       in ? dz + (((size_t)img * h + yy) * w + xx) * kC + q * 8 : dz, in);
-        }
-        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-        umma::fence_smem_to_async();
-        umma::fence_before_sync();
-        __syncthreads();
-        umma::fence_after_sync();
-        if (tid == 0) {
-            const uint32_t a0 = umma::smem_addr(sAct), b0 = umma::smem_addr(sDz);
-#pragma unroll 1
-            for (int r = 0; r < rows; ++r)
-#pragma unroll 1
-                for (int s = 0; s < steps; ++s) {
-                    const uint64_t bd = umma::desc(b0 + r * kSlot + s * 256, 128, kLbo);
-#pragma unroll
-                    for (int dx = 0; dx < 3; ++dx)
-                        umma::mma(tmem + 32 * dx, umma::desc(a0 + r * kSlot + s * 256 + dx * 16, 128, kLbo), bd, idesc,
-                                  !(first && r == 0 && s == 0));
-                }
-            umma::commit(&mbar);
-        }
-        for (int i = tid; i < rows * steps * 64; i += kWThreads) {
-            const int px = (i >> 2) % (16 * steps), r = (i >> 2) / (16 * steps);
-            const uint4 v = *reinterpret_cast<const uint4 *>(sDz + r * kSlot + (tid & 3) * kLbo + px * 16);
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                bsum[2 * e] += __uint_as_float(u[e] << 16);
-                bsum[2 * e + 1] += __uint_as_float(u[e] & 0xffff0000u);
+        const int rows = min(kWRowsT, h - y0), px = (min(kTilePx, w - x0) + 15) & ~15;
+        for (int r = 0; r < rows + 2; ++r) {
+            const int yy = y0 + r - 1;
+            const bool yin = yy >= 0 && yy < h;
+            const bf16 *src = act + ((long long)img * h + yy) * w * kC + q * 8;
+            for (int i = p0; i < px + 2; i += kWThreads / 4) {
+                const int xx = x0 - 1 + i;
+                const bool in = yin && xx >= 0 && xx < w;
+                cp_async16(buf + r * kSlot + q * kLbo + i * 16, in ? src + (long long)xx * kC : act, in);
             }
         }
+        for (int r = 0; r < rows; ++r) {
+            const bf16 *src = dz + ((long long)img * h + y0 + r) * w * kC + q * 8;
+            for (int i = p0; i < px; i += kWThreads / 4)
+                cp_async16(buf + kWAct + r * kSlot + q * kLbo + i * 16, x0 + i < w ? src + (long long)(x0 + i) * kC : dz,
+                           x0 + i < w);
+        }
+    };
+    uint32_t phase = 0;
+    bool first = true, ok = true;
+    float bsum[8] = {};   // channels 8 q ..
+    auto wait_mma = [&]() {
         const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase));
         phase ^= 1;
         if (!got) {
             ok = false;
             if (tid == 0) record_error(err, WV_ERR_TIMEOUT);
-            break;
+        }
+    };
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        if (!first) wait_mma();
+        if (!ok) break;
+        load(it);
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        umma::fence_smem_to_async();
+        umma::fence_before_sync();
+        __syncthreads();
+        umma::fence_after_sync();
+        const int x0 = (it % tx) * kTilePx, y0 = ((it / tx) % ty) * kWRowsT;
+        const int rows = min(kWRowsT, h - y0);
+        const int steps = (min(kTilePx, w - x0) + 15) / 16;   // K-steps of 16 pixels
+        if (warp < 3) {   // dx = warp: its own accumulator, its own issuing warp
+            const uint64_t a0 = umma::desc(umma::smem_addr(buf) + warp * 16, 128, kLbo);
+            const uint64_t b0 = umma::desc(umma::smem_addr(buf + kWAct), 128, kLbo);
+            const uint32_t d = tmem + 32 * warp;
+#pragma unroll 1
+            for (int r = 0; r < rows; ++r) {
+                const uint64_t ar = a0 + r * (kSlot >> 4), br = b0 + r * (kSlot >> 4);
+                if (umma::elect_one()) {
+#pragma unroll
+                    for (int s = 0; s < kTilePx / 16; ++s)
+                        if (s < steps) umma::mma(d, ar + 16 * s, br + 16 * s, idesc, !first || r > 0 || s > 0);
+                }
+                __syncwarp();
+            }
+            if (umma::elect_one()) umma::commit(&mbar);
+            __syncwarp();
         }
         first = false;
+        for (int r = 0; r < rows; ++r)
+            for (int i = p0; i < 16 * steps; i += kWThreads / 4) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(buf + kWAct + r * kSlot + q * kLbo + i * 16);
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    bsum[2 * e] += __uint_as_float(u[e] << 16);
+                    bsum[2 * e + 1] += __uint_as_float(u[e] & 0xffff0000u);
+                }
+            }
     }
+    if (!first && ok) wait_mma();
     if (!first && ok) {
         // the accumulators, reordered to the gradient's [co][ci][tap] in the
         // operand buffers (the MMAs have completed), then one coalesced pass
@@ -643,79 +680,95 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restri
 // cores, in fp32: G[tap][c] = sum over pixels q of T[q][c] P[q + tap - 1],
 // with T the layer's 32-channel tensor and P its one-channel plane.  First
 // layer: T = dZ, P = the input, tap as is; last layer: T = the input, P = dZ,
-// tap flipped (T[p + tap - 1] P[p] = T[q] P[q - (tap - 1)]).  A half warp walks
-// along a run of kERun pixels, each lane with two channels (one 4-byte load a
-// pixel) and the 3 x 3 window of P sliding in registers: 3 loads and 18 FMAs
-// a pixel, about 25 instructions per two pixels.  66 us for 16 x 256^2
-// pixels; the form staged in shared memory, with two loads per FMA, took 138
-// and 153 us.
-constexpr int kERun = 32;        // pixels per half warp and work item
+// tap flipped (T[p + tap - 1] P[p] = T[q] P[q - (tap - 1)]).  Four lanes hold a
+// pixel's channels (one 16-byte load each) and walk along a run of a row, eight
+// runs side by side in a warp, with the 3 x 3 window of P sliding in registers:
+// 4 loads and 36 packed FMAs for 8 pixels.  46 us for 16 x 256^2 pixels; staged
+// in shared memory, with two loads per FMA, it took 138 and 153 us.
 constexpr int kEWarps = 8;
+constexpr int kERunMax = 33;     // pixels per run, a multiple of the window's 3 columns
 
-__global__ void __launch_bounds__(32 * kEWarps) k_wgrad_edge(const float *__restrict__ plane,
-                                                            const bf16 *__restrict__ act, int first_layer, int n, int h,
-                                                            int w, float *dW, float *db) {
-    __shared__ float sum[kC * 9 + kC];   // [c][tap], then the bias
-    const int tid = threadIdx.x, lane = tid & 31, half = lane >> 4, c = 2 * (lane & 15);
-    for (int i = tid; i < kC * 10; i += 32 * kEWarps) sum[i] = 0.f;
-    __syncthreads();
-    float acc0[9] = {}, acc1[9] = {}, b0 = 0.f, b1 = 0.f;
-    const int runs = (w + 2 * kERun - 1) / (2 * kERun);
+__global__ void __launch_bounds__(32 * kEWarps, 2) k_wgrad_edge(const float *__restrict__ plane,
+                                                               const bf16 *__restrict__ act, int first_layer, int n, int h,
+                                                               int w, int run, int runs, float *dW, float *db) {
+    __shared__ float sum[kEWarps][kC * 10];   // [c][tap], then the bias
+    const int tid = threadIdx.x, lane = tid & 31, q = lane & 3, warp = tid >> 5;
+    float2 acc[9][4] = {}, bias[4] = {};
+    float centre = 0.f;
     const int total = n * h * runs;
-    for (int it = blockIdx.x * kEWarps + (tid >> 5); it < total; it += gridDim.x * kEWarps) {
+    for (int it = blockIdx.x * kEWarps + warp; it < total; it += gridDim.x * kEWarps) {
         const int y = (it / runs) % h, img = it / (runs * h);
-        const int xa = (it % runs) * 2 * kERun + half * kERun;
+        const int xa = ((it % runs) * 8 + (lane >> 2)) * run, xe = min(xa + run, w);
         const float *row = plane + ((size_t)img * h + y) * w;
-        const uint32_t *t = reinterpret_cast<const uint32_t *>(act + ((size_t)img * h + y) * w * kC + c);
+        const uint4 *t = reinterpret_cast<const uint4 *>(act + ((size_t)img * h + y) * w * kC) + q;
         const bool up = y > 0, dn = y + 1 < h;
         auto load = [&](int x, float (&v)[3]) {
-            const bool in = x >= 0 && x < w;
+            const bool in = (unsigned)x < (unsigned)w;
             v[0] = in && up ? __ldg(row - w + x) : 0.f;
             v[1] = in ? __ldg(row + x) : 0.f;
             v[2] = in && dn ? __ldg(row + w + x) : 0.f;
         };
-        float p0[3], p1[3];
-        load(xa - 1, p0);
-        load(xa, p1);
-#pragma unroll 4
-        for (int k = 0; k < kERun; ++k) {
-            const int x = xa + k;
-            float p2[3];
-            load(x + 1, p2);
-            const uint32_t u = x < w ? __ldg(t + (size_t)x * (kC / 2)) : 0u;
-            const float t0 = __uint_as_float(u << 16), t1 = __uint_as_float(u & 0xffff0000u);
+        float p[3][3];   // window columns x - 1, x, x + 1 (rotating)
+        load(xa - 1, p[0]);
+        load(xa, p[1]);
+#pragma unroll 1
+        for (int k0 = 0; k0 < run; k0 += 3)
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                acc0[3 * dy] = fmaf(t0, p0[dy], acc0[3 * dy]);
-                acc1[3 * dy] = fmaf(t1, p0[dy], acc1[3 * dy]);
-                acc0[3 * dy + 1] = fmaf(t0, p1[dy], acc0[3 * dy + 1]);
-                acc1[3 * dy + 1] = fmaf(t1, p1[dy], acc1[3 * dy + 1]);
-                acc0[3 * dy + 2] = fmaf(t0, p2[dy], acc0[3 * dy + 2]);
-                acc1[3 * dy + 2] = fmaf(t1, p2[dy], acc1[3 * dy + 2]);
+            for (int r = 0; r < 3; ++r) {
+                const int x = xa + k0 + r;
+                load(x + 1, p[(r + 2) % 3]);
+                const uint4 u = x < xe ? __ldg(t + 4 * (size_t)x) : make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
+                float2 tv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    tv[e] = make_float2(__uint_as_float(uw[e] << 16), __uint_as_float(uw[e] & 0xffff0000u));
+                    if (first_layer) bias[e] = __fadd2_rn(bias[e], tv[e]);
+                }
+                if (x < xe) centre += p[(r + 1) % 3][1];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float pv = p[(r + k % 3) % 3][k / 3];
+                    const float2 p2 = make_float2(pv, pv);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[k][e] = __ffma2_rn(tv[e], p2, acc[k][e]);
+                }
             }
-            // bias: the sum of dZ (the tensor, or the plane's centre)
-            b0 += first_layer ? t0 : (x < w ? p1[1] : 0.f);
-            b1 += t1;
+    }
+    // over the warp's eight runs, then over the CTA's warps
+    auto reduce = [&](float v) {
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) {
-                p0[dy] = p1[dy];
-                p1[dy] = p2[dy];
+        for (int o = 4; o < 32; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int tap = first_layer ? k : 8 - k;
+            const float s0 = reduce(acc[k][e].x), s1 = reduce(acc[k][e].y);
+            if (lane < 4) {
+                sum[warp][(8 * q + 2 * e) * 9 + tap] = s0;
+                sum[warp][(8 * q + 2 * e + 1) * 9 + tap] = s1;
             }
         }
+        const float b0 = reduce(bias[e].x), b1 = reduce(bias[e].y);
+        if (lane < 4) {
+            sum[warp][kC * 9 + 8 * q + 2 * e] = b0;
+            sum[warp][kC * 9 + 8 * q + 2 * e + 1] = b1;
+        }
     }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int tap = first_layer ? k : 8 - k;
-        const float s0 = acc0[k] + __shfl_xor_sync(0xffffffffu, acc0[k], 16);
-        const float s1 = acc1[k] + __shfl_xor_sync(0xffffffffu, acc1[k], 16);
-        atomicAdd(&sum[(c + half) * 9 + tap], half ? s1 : s0);
-    }
-    b0 += __shfl_xor_sync(0xffffffffu, b0, 16);
-    b1 += __shfl_xor_sync(0xffffffffu, b1, 16);
-    atomicAdd(&sum[kC * 9 + c + half], half ? b1 : b0);
+    centre = reduce(centre);
+    if (!first_layer && lane == 0) sum[warp][kC * 9] = centre;
     __syncthreads();
-    for (int i = tid; i < kC * 9; i += 32 * kEWarps) atomicAdd(dW + i, sum[i]);   // dW0[co][0][tap], dW4[0][ci][tap]
-    if (tid < (first_layer ? kC : 1)) atomicAdd(db + tid, sum[kC * 9 + tid]);
+    // dW0[co][0][tap], dW4[0][ci][tap]; the bias gradient is the sum of dZ:
+    // the tensor's (first layer) or the plane's (last layer)
+    for (int i = tid; i < kC * 9 + (first_layer ? kC : 1); i += 32 * kEWarps) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kEWarps; ++k) v += sum[k][i];
+        atomicAdd(i < kC * 9 ? dW + i : db + i - kC * 9, v);
+    }
 }
 
 // bf16 B operands from the fp32 master parameters (one thread per element).
@@ -865,7 +918,7 @@ cudaError_t launch_net(NetArgs &a, cudaStream_t cs) {
     if (e != cudaSuccess) return e;
     a.seg = seg_rows(a.n, a.h, a.w, BWD ? 3 : 4);
     const long long tasks = (long long)a.n * ((a.w + kTileOut - 1) / kTileOut) * ((a.h + a.seg - 1) / a.seg);
-    k_net<BWD><<<(int)std::min<long long>(tasks, sm_count()), kNetThreads, kNetSmem, cs>>>(a);
+    k_net<BWD><<<(int)std::min<long long>(tasks, sm_count()), net_threads(BWD), kNetSmem, cs>>>(a);
     return cudaGetLastError();
 }
 
@@ -881,9 +934,12 @@ cudaError_t launch_wgrad_mid(const bf16 *act, const bf16 *dz, int n, int h, int 
 
 cudaError_t launch_wgrad_edge(const float *plane, const bf16 *act, int first, int n, int h, int w, float *dW,
                               float *db, cudaStream_t cs) {
-    const int total = n * h * ((w + 2 * kERun - 1) / (2 * kERun));
+    // equal runs that cover a row with the fewest warps
+    const int runs = (w + 8 * kERunMax - 1) / (8 * kERunMax);
+    const int run = 3 * ((w + 24 * runs - 1) / (24 * runs));
+    const int total = n * h * runs;
     const int grid = std::max(1, std::min((total + kEWarps - 1) / kEWarps, 2 * sm_count()));
-    k_wgrad_edge<<<grid, 32 * kEWarps, 0, cs>>>(plane, act, first, n, h, w, dW, db);
+    k_wgrad_edge<<<grid, 32 * kEWarps, 0, cs>>>(plane, act, first, n, h, w, run, runs, dW, db);
     return cudaGetLastError();
 }
 

@@ -58,6 +58,16 @@ __device__ __forceinline__ void tmem_free(uint32_t taddr) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(COLS));
 }
 
+// True for one lane of a converged warp.  MMAs are issued inside
+// `if (elect_one())` by warps whose control flow and operands are uniform:
+// the operands then stay in uniform registers (behind `threadIdx.x == 0` an
+// MMA took over 150 cycles to issue).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r != 0;
+}
+
 // D[tmem] (+)= A[desc] * B[desc]^T, issued by one thread.
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
     asm volatile(
