@@ -198,12 +198,193 @@ __device__ __forceinline__ void resample_run(const ResampleArgs &a, int i, int j
     }
 }
 
-__global__ void k_resample(ResampleArgs a) {
-    resample_run(a, kPx * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y * blockDim.y + threadIdx.y);
+// ---- RGBA of projected positions --------------------------------------------
+//
+// The path of every viewport decode, written for instruction count and L1
+// wavefronts, which bound it (a pixel reads 4 luma bytes and 4 chroma words
+// that sit in L1 or L2):
+//   - a warp covers 16 x 4 pixels at a time, lane (x, y) = (lane % 8,
+//     lane / 8) taking pixels x and x + 8: a gather of 32 lanes then touches
+//     about half the 128-byte lines that 32 adjacent pixel pairs of one row
+//     do (rows of the viewport run diagonally through the frame);
+//   - the two pixels are projected in packed fp32x2 arithmetic (each element
+//     rounds as the scalar operations of project_px);
+//   - positions two pixels inside the plane take a path without wrap and
+//     clamp for luma and chroma together; the taps of a row share addresses,
+//     and with chroma groups the two taps of a row come out of two words with
+//     one funnel shift and one dot product per component.
+// RESAMPLEWHY
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// wv_atan2 of two (y, x) pairs; XPOS: x is not negative.
+template <bool XPOS>
+__device__ __forceinline__ float2 atan2_pair(float2 y, float2 x) {
+    const float ax0 = fabsf(x.x), ay0 = fabsf(y.x), ax1 = fabsf(x.y), ay1 = fabsf(y.y);
+    const float mx0 = fmaxf(ax0, ay0), mx1 = fmaxf(ax1, ay1);
+    float r0, r1;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(mx0));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(mx1));
+    float2 t = __fmul2_rn(make_float2(fminf(ax0, ay0), fminf(ax1, ay1)), make_float2(r0, r1));
+    if (!(mx0 > 0.0f)) t.x = 0.0f;
+    if (!(mx1 > 0.0f)) t.y = 0.0f;
+    const float2 u = __fmul2_rn(t, t);
+    float2 p = f2(-0.0017539301188662648f);
+    p = __ffma2_rn(p, u, f2(0.010726944543421268f));
+    p = __ffma2_rn(p, u, f2(-0.030804596841335297f));
+    p = __ffma2_rn(p, u, f2(0.05755210295319557f));
+    p = __ffma2_rn(p, u, f2(-0.0837731584906578f));
+    p = __ffma2_rn(p, u, f2(0.1094203069806099f));
+    p = __ffma2_rn(p, u, f2(-0.142619326710701f));
+    p = __ffma2_rn(p, u, f2(0.1999826580286026f));
+    p = __ffma2_rn(p, u, f2(-0.3333328366279602f));
+    p = __ffma2_rn(p, u, f2(1.0f));
+    float2 r = __fmul2_rn(p, t);
+    const float2 c = __fadd2_rn(neg2(r), f2(1.5707963267948966f));
+    if (ay0 > ax0) r.x = c.x;
+    if (ay1 > ax1) r.y = c.y;
+    if (!XPOS) {
+        const float2 d = __fadd2_rn(neg2(r), f2(3.141592653589793f));
+        if (x.x < 0.0f) r.x = d.x;
+        if (x.y < 0.0f) r.y = d.y;
+    }
+    return make_float2(copysignf(r.x, y.x), copysignf(r.y, y.y));
+}
+
+// project_px of pixels (i, j) and (i + 8, j).  The rotation has no roll
+// (r[3] = 0): the ray's y does not depend on the column.
+__device__ __forceinline__ void project_pair(const View &v, int i, int j, float2 &u, float2 &w) {
+    const float2 xc = __fadd2_rn(make_float2((float)i, (float)(i + 8)), f2(0.5f));
+    const float2 xn = __fmul2_rn(__ffma2_rn(xc, f2(v.sx), f2(-1.0f)), f2(v.t));
+    const float yn = __fmul_rn(fmaf(-((float)j + 0.5f), v.sy, 1.0f), v.t);
+    const float2 dx = __ffma2_rn(f2(v.r[0]), xn, f2(fmaf(v.r[1], yn, v.r[2])));
+    const float2 dy = f2(fmaf(v.r[4], yn, v.r[5]));
+    const float2 dz = __ffma2_rn(f2(v.r[6]), xn, f2(fmaf(v.r[7], yn, v.r[8])));
+    const float2 q = __ffma2_rn(dx, dx, __fmul2_rn(dz, dz));
+    const float2 h = make_float2(sqrtf(q.x), sqrtf(q.y));
+    u = __ffma2_rn(atan2_pair<false>(dx, dz), f2(v.ku), f2(v.cu));
+    w = __ffma2_rn(atan2_pair<true>(dy, h), f2(v.kv), f2(v.cv));
+}
+
+// Rounded blend of two rows' horizontal sums.
+__device__ __forceinline__ int blend_rows(int top, int bot, int fy) {
+    return ((256 - fy) * top + (fy * bot + 32768)) >> 16;
+}
+
+// Channel layouts of a stream: grey, chroma planes, chroma in alternating
+// 4-sample groups.
+enum Chroma { kGrey = 0, kPlanar = 1, kGroups = 2 };
+
+// One pixel at luma position (u, w) at least two pixels inside the plane
+// (its chroma taps then lie inside theirs).
+template <int CH, bool C420>
+__device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int Y, float uc, float vc) {
+    const int fx = X & 255, fy = Y & 255;
+    const unsigned W = a.w[0];
+    const uint8_t *p = a.plane[0] + (unsigned)((Y >> 8) * (int)W + (X >> 8));
+    const uint8_t *q = p + W;
+    const int y = blend_rows((256 - fx) * __ldg(p) + fx * __ldg(p + 1), (256 - fx) * __ldg(q) + fx * __ldg(q + 1), fy);
+    if constexpr (CH == kGrey) {
+        return rgba_word(to_rgba(y, 128, 128));
+    } else {
+        int Xc = X, Yc = Y;
+        if constexpr (C420) {
+            Xc = __float2int_rd(fmaf(uc, 256.0f, 0.5f));
+            Yc = __float2int_rd(fmaf(vc, 256.0f, 0.5f));
+        }
+        const int gx = Xc & 255, gy = Yc & 255;
+        const unsigned Wc = a.w[1], e = (unsigned)((Yc >> 8) * (int)Wc + (Xc >> 8));
+        int cb, cr;
+        if constexpr (CH == kGroups) {
+            // rows are whole groups: the next row is 2 Wc bytes on
+            const uint8_t *g0 = a.plane[1] + 8u * (e >> 2), *g1 = a.plane[1] + 8u * ((e + 1) >> 2);
+            const uint2 t0 = __ldg(reinterpret_cast<const uint2 *>(g0)), t1 = __ldg(reinterpret_cast<const uint2 *>(g1));
+            const uint2 b0 = __ldg(reinterpret_cast<const uint2 *>(g0 + 2 * Wc)), b1 = __ldg(reinterpret_cast<const uint2 *>(g1 + 2 * Wc));
+            // bytes k, k + 1 of the two groups side by side (taps of one
+            // group: both words are that group, so byte k + 1 <= 3)
+            const int sh = 8 * (e & 3);
+            const unsigned wt = (unsigned)(256 - gx) | ((unsigned)gx << 16);
+            const int cbt = __dp2a_lo(wt, __funnelshift_r(t0.x, t1.x, sh), 0u), cbb = __dp2a_lo(wt, __funnelshift_r(b0.x, b1.x, sh), 0u);
+            const int crt = __dp2a_lo(wt, __funnelshift_r(t0.y, t1.y, sh), 0u), crb = __dp2a_lo(wt, __funnelshift_r(b0.y, b1.y, sh), 0u);
+            cb = blend_rows(cbt, cbb, gy);
+            cr = blend_rows(crt, crb, gy);
+        } else {
+            const uint8_t *p1 = a.plane[1] + e, *p2 = a.plane[2] + e;
+            const uint8_t *q1 = p1 + Wc, *q2 = p2 + Wc;
+            cb = blend_rows((256 - gx) * __ldg(p1) + gx * __ldg(p1 + 1), (256 - gx) * __ldg(q1) + gx * __ldg(q1 + 1), gy);
+            cr = blend_rows((256 - gx) * __ldg(p2) + gx * __ldg(p2 + 1), (256 - gx) * __ldg(q2) + gx * __ldg(q2 + 1), gy);
+        }
+        // to_rgba with the constants gathered, saturating packs
+        const int rr = (y * 65536 + (kRCr * cr + (32768 - 128 * kRCr))) >> 16;
+        const int gg = (y * 65536 + (-kGCb * cb + (-kGCr * cr + (32768 + 128 * (kGCb + kGCr))))) >> 16;
+        const int bb = (y * 65536 + (kBCb * cb + (32768 - 128 * kBCb))) >> 16;
+        uint32_t hi, d;
+        asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(255), "r"(bb));
+        asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(gg), "r"(rr), "r"(hi));
+        return d;
+    }
+}
+
+constexpr int kPatchW = 64, kPatchH = 16;   // pixels per CTA: warps 4 x 2, two row groups each
+
+template <int CH, bool C420>
+__device__ __forceinline__ void resample_patch(const ResampleArgs &a, int bx, int by) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = bx * kPatchW + (warp & 3) * 16 + (lane & 7);
+    const int W = a.w[0], r0 = a.v.row0, rn = a.v.rows;
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        const int j = by * kPatchH + (warp >> 2) * 8 + 4 * k + (lane >> 3);
+        if (i >= a.v.out_w || j >= a.v.out_h) return;
+        float2 u, w;
+        project_pair(a.v, i, j, u, w);
+        const float2 X = __ffma2_rn(u, f2(256.0f), f2(0.5f)), Y = __ffma2_rn(w, f2(256.0f), f2(0.5f));
+        float2 uc = u, vc = w;
+        if (C420) {
+            uc = __ffma2_rn(__fadd2_rn(u, f2(0.5f)), f2(0.5f), f2(-0.5f));
+            vc = __ffma2_rn(__fadd2_rn(w, f2(0.5f)), f2(0.5f), f2(-0.5f));
+        }
+        uint32_t *dst = reinterpret_cast<uint32_t *>(a.out + (size_t)j * a.pitch) + i;
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (m && i + 8 >= a.v.out_w) break;
+            const int Xi = __float2int_rd(m ? X.y : X.x), Yi = __float2int_rd(m ? Y.y : Y.x);
+            const bool in = (unsigned)((Xi >> 8) - 2) < (unsigned)(W - 6) && (unsigned)((Yi >> 8) - r0 - 2) < (unsigned)(rn - 6);
+            uint32_t c;
+            if (in) c = inside_px<CH, C420>(a, Xi, Yi, m ? uc.y : uc.x, m ? vc.y : vc.x);
+            else c = rgba_word(sample_px(a, m ? u.y : u.x, m ? w.y : w.x));
+            dst[8 * m] = c;
+        }
+    }
+}
+
+__device__ __forceinline__ void resample_any(const ResampleArgs &a, int bx, int by) {
+    if (a.planes != 3) resample_patch<kGrey, false>(a, bx, by);
+    else if (a.c_pair && a.c420) resample_patch<kGroups, true>(a, bx, by);
+    else if (a.c_pair) resample_patch<kGroups, false>(a, bx, by);
+    else if (a.c420) resample_patch<kPlanar, true>(a, bx, by);
+    else resample_patch<kPlanar, false>(a, bx, by);
+}
+
+template <int CH, bool C420>
+__global__ void __launch_bounds__(256) k_resample(ResampleArgs a) {
+    resample_patch<CH, C420>(a, blockIdx.x, blockIdx.y);
 }
 
 // Batch: one z-slice of the grid per request.
-__global__ void k_resample_batch(const RequestJob *__restrict__ reqs) {
+__global__ void __launch_bounds__(256) k_resample_batch(const RequestJob *__restrict__ reqs) {
+    const ResampleArgs &a = reqs[blockIdx.z].rs;
+    if ((int)blockIdx.x * kPatchW >= a.v.out_w || (int)blockIdx.y * kPatchH >= a.v.out_h) return;
+    resample_any(a, blockIdx.x, blockIdx.y);
+}
+
+// Caller-given positions, luma and chroma planes instead of RGBA, and (in
+// WV_CHECKED builds) every tap checked.
+__global__ void k_resample_general(ResampleArgs a) {
+    resample_run(a, kPx * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y * blockDim.y + threadIdx.y);
+}
+__global__ void k_resample_general_batch(const RequestJob *__restrict__ reqs) {
     const ResampleArgs &a = reqs[blockIdx.z].rs;
     resample_run(a, kPx * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y * blockDim.y + threadIdx.y);
 }
@@ -231,15 +412,28 @@ void launch_resample(const Geom &g, const View &v, uint8_t *const *recon, const 
     a.uv = uv;
     a.out = out;
     a.pitch = pitch;
-    dim3 block(32, 8);
-    dim3 grid((v.out_w + 32 * kPx - 1) / (32 * kPx), (v.out_h + 7) / 8);
-    k_resample<<<grid, block, 0, cs>>>(a);
+    if (uv || y_plane || kChecked) {
+        dim3 block(32, 8);
+        dim3 grid((v.out_w + 32 * kPx - 1) / (32 * kPx), (v.out_h + 7) / 8);
+        k_resample_general<<<grid, block, 0, cs>>>(a);
+        return;
+    }
+    const dim3 grid((v.out_w + kPatchW - 1) / kPatchW, (v.out_h + kPatchH - 1) / kPatchH);
+    if (a.planes != 3) k_resample<kGrey, false><<<grid, 256, 0, cs>>>(a);
+    else if (a.c_pair && a.c420) k_resample<kGroups, true><<<grid, 256, 0, cs>>>(a);
+    else if (a.c_pair) k_resample<kGroups, false><<<grid, 256, 0, cs>>>(a);
+    else if (a.c420) k_resample<kPlanar, true><<<grid, 256, 0, cs>>>(a);
+    else k_resample<kPlanar, false><<<grid, 256, 0, cs>>>(a);
 }
 
 void launch_resample_batch(const RequestJob *reqs, int n, int max_w, int max_h, cudaStream_t cs) {
-    dim3 block(32, 8);
-    dim3 grid((max_w + 32 * kPx - 1) / (32 * kPx), (max_h + 7) / 8, n);
-    k_resample_batch<<<grid, block, 0, cs>>>(reqs);
+    if (kChecked) {
+        dim3 block(32, 8);
+        dim3 grid((max_w + 32 * kPx - 1) / (32 * kPx), (max_h + 7) / 8, n);
+        k_resample_general_batch<<<grid, block, 0, cs>>>(reqs);
+        return;
+    }
+    k_resample_batch<<<dim3((max_w + kPatchW - 1) / kPatchW, (max_h + kPatchH - 1) / kPatchH, n), 256, 0, cs>>>(reqs);
 }
 
 }  // namespace wv
