@@ -9,8 +9,11 @@
 // dead-zone quantiser q = sign(c) floor(|c| / step).  Blocks whose quantised
 // coefficients are all zero are omitted (Sec. 3.4 loads only stored blocks).
 #include <string.h>
+#include <unistd.h>
 
 #include <algorithm>
+#include <system_error>
+#include <thread>
 #include <type_traits>
 #include <vector>
 
@@ -432,6 +435,29 @@ cudaError_t transform_plane(const uint8_t *src, T *work, T *tmp, int w, int h, i
     return cudaGetLastError();
 }
 
+// Writes one byte of every page of the n bytes at p, which the caller is
+// about to overwrite, from several threads.  A caller's fresh buffer has no
+// pages yet, and the copy from the device would fault them in one at a time:
+// 104 MB took 3.9 ms, 0.6 into pages that are there.
+void touch_pages(char *p, size_t n) {
+    constexpr size_t kShare = size_t(4) << 20;   // bytes below which a thread costs more than its faults
+    const size_t page = (size_t)std::max(sysconf(_SC_PAGESIZE), 4096l);
+    const size_t parts = std::min<size_t>({n / kShare, 8, std::max(1u, std::thread::hardware_concurrency())});
+    if (parts < 2) return;
+    auto touch = [=](size_t lo, size_t hi) {
+        for (size_t i = lo; i < hi; i += page) *(volatile char *)(p + i) = 0;
+    };
+    std::thread t[8];
+    size_t started = 0;
+    try {
+        for (; started < parts - 1; ++started)
+            t[started] = std::thread(touch, n / parts * started, n / parts * (started + 1));
+    } catch (const std::system_error &) {   // no thread to be had: the copy faults the pages in
+    }
+    touch(n / parts * (parts - 1), n);
+    for (size_t i = 0; i < started; ++i) t[i].join();
+}
+
 template <typename T>
 int run(const Geom &g, const void *const *planes, char *base, const ScratchLayout &S, void *out,
         size_t cap, size_t *out_len, cudaStream_t cs) {
@@ -509,6 +535,7 @@ int run(const Geom &g, const void *const *planes, char *base, const ScratchLayou
     k_pack<<<dim3(g.nbpf, g.num_frames), 256, 0, cs>>>(coef_ptrs, desc, plane_w, plane_off, g.nbpf, flags,
                                                        g.block, payload);
     char *o = (char *)out;
+    touch_pages(o + payload_off, (size_t)nslots * bbytes);
     memset(o, 0, payload_off);
     StreamHeader h;
     memset(&h, 0, sizeof(h));
