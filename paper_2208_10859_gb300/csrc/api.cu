@@ -106,7 +106,9 @@ int stream_geoms(const wv_stream_desc &d, uint64_t n_payload, Geom *g, Geom *gsq
     if (rc != WV_OK) return rc;
     gsq->n_blocks = (int)std::min<uint64_t>(n_payload, 0x7fffffff);
     if (strip_eligible(d, n_payload)) {
-        const int rs = build_geom_strip(d, g);
+        const int strips = viewable_strips(d);
+        const int rs = strips <= kFineStrips ? build_geom_strip(d, g, 32, 32) : build_geom_strip(d, g);
+        g->halves = strips <= kFineStrips / 4;
         g->n_blocks = gsq->n_blocks;
         return rs;
     }
@@ -212,7 +214,7 @@ int check_image(const wv_image *o) {
 // reading LL_2 from the planes.
 cudaError_t launch_fine(wv_stream *s, const Bands &b, const float *const *ll2, uint8_t *const *out_u8,
                         float *f32, int f32_plane, const uint32_t *tiles, int *counters,
-                        cudaStream_t cs) {
+                        cudaStream_t cs, int all_plane = -1) {
     const Geom &g = active_geom(s);
     if (strip_mode(s)) {
         // into the stream's reconstruction planes: chroma in alternating Cb, Cr groups
@@ -221,25 +223,25 @@ cudaError_t launch_fine(wv_stream *s, const Bands &b, const float *const *ll2, u
         const bool pairs = own && recon_pairs(s);
         uint8_t *const outs[3] = {out_u8[0], out_u8[1], pairs ? out_u8[1] + 4 : out_u8[2]};
         return launch_decode_strips(g, s->payload, s->table, b, ll2, s->ll2_pitch, outs, f32, f32_plane, tiles,
-                                    counters, s->err, cs, pairs);
+                                    counters, s->err, cs, pairs, all_plane);
     }
     return launch_decode_fine(g, s->payload, s->table, b, ll2, s->ll2_pitch, out_u8, f32, f32_plane, tiles,
                               counters, s->err, cs);
 }
 
 cudaError_t run_decode(wv_stream *s, const Bands &b, uint8_t *const *out_u8, float *f32,
-                       int f32_plane) {
+                       int f32_plane, int all_plane = -1) {
     const Geom &g = active_geom(s);
     cudaError_t e;
     if (split_mode(s)) {
         prof_begin(s, kKCoarse);
         e = launch_decode_coarse(g, s->payload, s->table, b, s->ll2, s->ll2_pitch, s->ctiles,
-                                 s->counters + 1, s->err, s->cs);
+                                 s->counters + 1, s->err, s->cs, all_plane);
         prof_end(s);
         if (e != cudaSuccess) return e;
         const float *ll2c[3] = {s->ll2[0], s->ll2[1], s->ll2[2]};
         prof_begin(s, kKFine);
-        e = launch_fine(s, b, ll2c, out_u8, f32, f32_plane, s->tiles, s->counters, s->cs);
+        e = launch_fine(s, b, ll2c, out_u8, f32, f32_plane, s->tiles, s->counters, s->cs, all_plane);
         prof_end(s);
         return e;
     }
@@ -629,13 +631,22 @@ int build_geom_rect(const wv_stream_desc &d, Geom *g, int tw, int th, int ctile)
     return build_geom_tiles(d, g, tw, th, 0, ctile);
 }
 
-// The strip kernel decodes levels 2 and 1 of dead-zone streams of three or
-// more levels (LL_2 from the coarse pass; taking it from the LL band of
-// two-level streams in the same loop cost 5 % in spilled registers) and
-// addresses the payload with 32-bit element offsets.
+// The strip kernel decodes levels 2 and 1 of streams of three or more levels
+// (LL_2 from the coarse pass; taking it from the LL band of two-level streams
+// in the same loop cost 5 % in spilled registers) and addresses the payload
+// with 32-bit element offsets.
 bool strip_eligible(const wv_stream_desc &d, uint64_t n_payload) {
-    return d.levels >= 3 && d.quant == 0 &&
+    return d.levels >= 3 && (d.quant == 0 || d.wavelet == WV_WAVELET_97) &&
            n_payload * (uint64_t)d.block * (uint64_t)d.block < (1ull << 32);
+}
+
+int viewable_strips(const wv_stream_desc &d) {
+    long long n = 0;
+    for (int p = 0; p < d.planes; ++p) {
+        const int sub = p > 0 && d.chroma_420 ? 2 : 1;
+        n += ((d.width / sub + kStripW - 1) / kStripW) * (long long)((d.height / sub + 63) / 64);
+    }
+    return (int)std::min<long long>(n / (d.stereo ? 2 : 1), 0x7fffffff);
 }
 
 int build_geom_strip(const wv_stream_desc &d, Geom *g, int th, int ctile) {
@@ -936,14 +947,14 @@ int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float)
     if (!s || frame < 0 || frame >= s->g.num_frames || plane < 0 || plane >= s->g.planes)
         return WV_ERR_ARG;
     if (!dptr && as_float) return WV_ERR_ARG;
-    // the strip fine pass writes 8-bit samples only: float output runs the
+    // float output of streams the float strip kernels do not take runs the
     // square-tile passes (the same arithmetic per sample)
     struct ModeGuard {
         wv_stream *s;
         int saved;
         ~ModeGuard() { s->decode_mode = saved; }
     } guard{s, s->decode_mode};
-    if (as_float && strip_mode(s)) s->decode_mode = 2;
+    if (as_float && strip_mode(s) && !strip_float_supported(s->g)) s->decode_mode = 2;
     const Geom &g = active_geom(s);
     uint8_t *outs[3] = {s->recon[0], s->recon[1], s->recon[2]};
     float *f32 = nullptr;
@@ -951,9 +962,12 @@ int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float)
         if (as_float) f32 = (float *)dptr;
         else outs[plane] = (uint8_t *)dptr;
     }
-    launch_all_tiles(g, plane, s->tiles, s->counters, s->cs);
-    if (split_mode(s)) launch_all_ctiles(g, plane, s->ctiles, s->counters, s->cs);
-    cudaError_t e = run_decode(s, stream_bands(s, frame), outs, f32, as_float ? plane : -1);
+    // strips: every tile of the plane, without lists (their count only serves
+    // the profile)
+    const int all_plane = strip_mode(s) ? plane : -1;
+    if (all_plane < 0 || s->prof) launch_all_tiles(g, plane, s->tiles, s->counters, s->cs);
+    if (all_plane < 0 && split_mode(s)) launch_all_ctiles(g, plane, s->ctiles, s->counters, s->cs);
+    cudaError_t e = run_decode(s, stream_bands(s, frame), outs, f32, as_float ? plane : -1, all_plane);
     mark_sets_used(s);
     if (!dptr) {   // set 0's reconstruction now holds the decode (for wv_resample_at)
         s->cur = 0;

@@ -210,7 +210,7 @@ __global__ void k_select_tiles(Geom g, const uint32_t *__restrict__ tile_gen,
     // edge strips are listed as two half strips (their reflected columns
     // make them the slowest tiles; halves halve their latency)
     const bool split = sel && !coarse && g.strip &&
-                       !strip_interior((int)(entry & 0x3fff), g.p[(entry >> 28) & 3].w) &&
+                       (g.halves || !strip_interior((int)(entry & 0x3fff), g.p[(entry >> 28) & 3].w)) &&
                        (int)((entry >> 14) & 0x3fff) * g.th + g.th / 2 < g.p[(entry >> 28) & 3].h;
     if (split) entry |= kHalfStrip;
     // warps straddling the two ranges: every call is made by all lanes
@@ -247,7 +247,7 @@ __global__ void k_select_batch(const SurfaceJob *__restrict__ surfs, BatchLists 
     const int c = s.cls;
     // strip surfaces: fine tiles to the strip list, edge strips as two halves
     const bool st = sel && !is_coarse && s.strip;
-    const bool split = st && !strip_interior((int)(e.y & 0x3fff), g.p[(e.y >> 28) & 3].w) &&
+    const bool split = st && (g.halves || !strip_interior((int)(e.y & 0x3fff), g.p[(e.y >> 28) & 3].w)) &&
                        (int)((e.y >> 14) & 0x3fff) * g.th + g.th / 2 < g.p[(e.y >> 28) & 3].h;
     if (split) e.y |= kHalfStrip;
     append2(st, e, lists.strip[c], &ctr[4 * c + 3]);

@@ -769,12 +769,16 @@ __device__ __forceinline__ void decode_one(const TileArgs &a, uint32_t e, float 
 }
 
 template <int WAV, int NB, int QM, bool CHK = false>
-__global__ void __launch_bounds__(kThreads, 2) k_tiles(TileArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) k_tiles(TileArgs a, AllTiles all) {
     extern __shared__ __align__(16) float smem[];
     float *A = smem;
     float *P = smem + a.a_floats;
-    const int count = *(volatile const int *)a.count;
-    for (int ti = blockIdx.x; ti < count; ti += gridDim.x) decode_one<WAV, NB, false, QM, CHK>(a, a.tiles[ti], A, P);
+    int count = all.n;
+    if (count == 0) count = *(volatile const int *)a.count;
+    for (int ti = blockIdx.x; ti < count; ti += gridDim.x) {
+        const uint32_t e = all.n ? all.entry(ti) : a.tiles[ti];
+        decode_one<WAV, NB, false, QM, CHK>(a, e, A, P);
+    }
 }
 
 // ---- batched decode: one persistent launch over all surfaces ---------------
@@ -926,11 +930,11 @@ void fill_tile_scales(TileArgs &a) {
 namespace {
 
 template <int WAV, int NB, int QM = 0, bool CHK = kChecked>
-cudaError_t launch_t(const TileArgs &a, int grid, int threads, cudaStream_t cs) {
+cudaError_t launch_t(const TileArgs &a, const AllTiles &all, int grid, int threads, cudaStream_t cs) {
     const int smem = (a.a_floats + a.p_floats) * 4;
     cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_tiles<WAV, NB, QM, CHK>), smem);
     if (e != cudaSuccess) return e;
-    k_tiles<WAV, NB, QM, CHK><<<grid, threads, smem, cs>>>(a);
+    k_tiles<WAV, NB, QM, CHK><<<grid, threads, smem, cs>>>(a, all);
     return cudaGetLastError();
 }
 
@@ -950,7 +954,7 @@ cudaError_t launch_batch_t(const SurfaceJob *surfs, const uint2 *coarse, const u
     return cudaGetLastError();
 }
 
-cudaError_t launch_args(TileArgs &a, cudaStream_t cs) {
+cudaError_t launch_args(TileArgs &a, cudaStream_t cs, const AllTiles &all = AllTiles{}) {
     fill_tile_scales(a);
     // the coarse pass has few, small tiles: 4-warp CTAs, four per SM (its
     // latency, not its work, sets its duration); tile passes: 8 warps, two
@@ -964,48 +968,48 @@ cudaError_t launch_args(TileArgs &a, cudaStream_t cs) {
         if (a.g.quant != 0 || a.g.dz_t) return cudaErrorInvalidValue;
         if (a.g.wavelet == WV_WAVELET_97) {
             switch (nb) {
-            case 1: return launch_t<1, 1, 0, true>(a, grid, threads, cs);
-            case 2: return launch_t<1, 2, 0, true>(a, grid, threads, cs);
-            case 3: return launch_t<1, 3, 0, true>(a, grid, threads, cs);
-            default: return launch_t<1, 4, 0, true>(a, grid, threads, cs);
+            case 1: return launch_t<1, 1, 0, true>(a, all, grid, threads, cs);
+            case 2: return launch_t<1, 2, 0, true>(a, all, grid, threads, cs);
+            case 3: return launch_t<1, 3, 0, true>(a, all, grid, threads, cs);
+            default: return launch_t<1, 4, 0, true>(a, all, grid, threads, cs);
             }
         }
         switch (nb) {
-        case 1: return launch_t<0, 1, 0, true>(a, grid, threads, cs);
-        case 2: return launch_t<0, 2, 0, true>(a, grid, threads, cs);
-        case 3: return launch_t<0, 3, 0, true>(a, grid, threads, cs);
-        default: return launch_t<0, 4, 0, true>(a, grid, threads, cs);
+        case 1: return launch_t<0, 1, 0, true>(a, all, grid, threads, cs);
+        case 2: return launch_t<0, 2, 0, true>(a, all, grid, threads, cs);
+        case 3: return launch_t<0, 3, 0, true>(a, all, grid, threads, cs);
+        default: return launch_t<0, 4, 0, true>(a, all, grid, threads, cs);
         }
     }
     if (a.g.quant == 1) {   // paper-faithful byte quantiser (9/7 only)
         switch (nb) {
-        case 1: return launch_t<1, 1, 1>(a, grid, threads, cs);
-        case 2: return launch_t<1, 2, 1>(a, grid, threads, cs);
-        case 3: return launch_t<1, 3, 1>(a, grid, threads, cs);
-        default: return launch_t<1, 4, 1>(a, grid, threads, cs);
+        case 1: return launch_t<1, 1, 1>(a, all, grid, threads, cs);
+        case 2: return launch_t<1, 2, 1>(a, all, grid, threads, cs);
+        case 3: return launch_t<1, 3, 1>(a, all, grid, threads, cs);
+        default: return launch_t<1, 4, 1>(a, all, grid, threads, cs);
         }
     }
     if (a.g.wavelet == WV_WAVELET_97 && a.g.dz_t) {   // codes stored as 2q + sign(q)
         switch (nb) {
-        case 1: return launch_t<1, 1, 2>(a, grid, threads, cs);
-        case 2: return launch_t<1, 2, 2>(a, grid, threads, cs);
-        case 3: return launch_t<1, 3, 2>(a, grid, threads, cs);
-        default: return launch_t<1, 4, 2>(a, grid, threads, cs);
+        case 1: return launch_t<1, 1, 2>(a, all, grid, threads, cs);
+        case 2: return launch_t<1, 2, 2>(a, all, grid, threads, cs);
+        case 3: return launch_t<1, 3, 2>(a, all, grid, threads, cs);
+        default: return launch_t<1, 4, 2>(a, all, grid, threads, cs);
         }
     }
     if (a.g.wavelet == WV_WAVELET_97) {
         switch (nb) {
-        case 1: return launch_t<1, 1>(a, grid, threads, cs);
-        case 2: return launch_t<1, 2>(a, grid, threads, cs);
-        case 3: return launch_t<1, 3>(a, grid, threads, cs);
-        default: return launch_t<1, 4>(a, grid, threads, cs);
+        case 1: return launch_t<1, 1>(a, all, grid, threads, cs);
+        case 2: return launch_t<1, 2>(a, all, grid, threads, cs);
+        case 3: return launch_t<1, 3>(a, all, grid, threads, cs);
+        default: return launch_t<1, 4>(a, all, grid, threads, cs);
         }
     }
     switch (nb) {
-    case 1: return launch_t<0, 1>(a, grid, threads, cs);
-    case 2: return launch_t<0, 2>(a, grid, threads, cs);
-    case 3: return launch_t<0, 3>(a, grid, threads, cs);
-    default: return launch_t<0, 4>(a, grid, threads, cs);
+    case 1: return launch_t<0, 1>(a, all, grid, threads, cs);
+    case 2: return launch_t<0, 2>(a, all, grid, threads, cs);
+    case 3: return launch_t<0, 3>(a, all, grid, threads, cs);
+    default: return launch_t<0, 4>(a, all, grid, threads, cs);
     }
 }
 
@@ -1061,10 +1065,14 @@ cudaError_t launch_decode_tiles(const Geom &g, const int16_t *payload, const int
 // level 2) into float LL_2 planes (float bits of int values for 5/3).
 cudaError_t launch_decode_coarse(const Geom &g, const int16_t *payload, const int32_t *table,
                                  const Bands &bands, float *const *ll2, const int *ll2_pitch,
-                                 const uint32_t *tiles, const int *count, int *err, cudaStream_t cs) {
+                                 const uint32_t *tiles, const int *count, int *err, cudaStream_t cs,
+                                 int all_plane) {
     TileArgs a = base_args(g, payload, table, bands, err);
     a.l_top = g.levels;
     a.l_bot = 3;
+    AllTiles all{};
+    if (all_plane >= 0)   // every coarse tile of a plane
+        all = AllTiles{g.p[all_plane].ctiles_x * g.p[all_plane].ctiles_y, all_plane, g.p[all_plane].ctiles_x};
     a.tw = a.th = g.ctile;
     for (int p = 0; p < 3; ++p) {
         a.ll_out[p] = ll2[p];
@@ -1072,7 +1080,7 @@ cudaError_t launch_decode_coarse(const Geom &g, const int16_t *payload, const in
     }
     a.tiles = tiles;
     a.count = count;
-    return launch_args(a, cs);
+    return launch_args(a, cs, all);
 }
 
 // Levels 2 and 1 of the listed tiles, reading LL_2 from the planes written by

@@ -26,9 +26,10 @@
 // lanes 1..28 write the strip's 224 columns.  Vertically the first pairs
 // of a tile only warm the running state up (four pairs per level for 9/7).
 //
-// A strip touching the plane's left or right side (an edge strip) may be
-// listed as two half strips of th / 2 rows each: its reflected columns make
-// it the slowest tile, and the launch lasts as long as its slowest tile.
+// A strip touching the plane's left or right side (an edge strip), and in
+// small frames every strip, is listed as two half strips of th / 2 rows each:
+// its reflected columns make it the slowest tile, and the launch lasts as
+// long as its slowest tile.
 // The same strips of many decode targets run in one batched launch
 // (k_strip_batch), with foveation (Sec. 3.7) dropping the detail rows of
 // the cells outside its radii in the gather.
@@ -55,7 +56,6 @@ namespace wv {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kStripWarps = 4;          // warps (strip tiles in flight) per CTA
 constexpr int kRing = 8;                // LL_1 rows held per warp (two iterations + reflection)
 constexpr int kRingW = 136;             // floats per ring row (128 used + a lane 31 overrun)
 constexpr uint32_t kNone = 0xffffffffu; // absent block
@@ -91,11 +91,25 @@ __device__ __forceinline__ float to_f(T v) {
 // codes held as t = 2q + sign(q) (c = t step / 2, scale s carries step / 2);
 // QM = 0: codes q (9/7: c = (2q + sign q) step / 2; 5/3: integer
 // reconstruction sign(q)(|q| step + floor(step / 2))).  5/3 frames combine by
-// the inverse S-transform.
+// the inverse S-transform.  QM = 1: the record format's byte quantiser, code +
+// 1 of a detail band (0: dropped), c = c_min + code times the plane's step of
+// that coefficient frame, s back to 8-bit units.
 template <int WAV, int NB, int QM>
-__device__ __forceinline__ void dq_word(const uint32_t (&w)[NB], const Bands &bd, float s, int st,
+__device__ __forceinline__ void dq_word(const uint32_t (&w)[NB], const Bands &bd, float s, int st, int plane,
                                         typename SV<WAV>::T &lo, typename SV<WAV>::T &hi) {
-    if constexpr (WAV == 1 && QM == 2 && NB == 1) {
+    if constexpr (QM == 1) {
+        float al = 0.f, ah = 0.f;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const float c0 = bd.qp[b][plane][1][0], d = bd.qp[b][plane][1][1];
+            const float sg = (b == 0 || bd.bit[b]) ? 1.f : -1.f;
+            const int ql = lo16(w[b]), qh = hi16(w[b]);
+            al = fmaf(sg, ql ? fmaf((float)(ql - 1), d, c0) : 0.f, al);
+            ah = fmaf(sg, qh ? fmaf((float)(qh - 1), d, c0) : 0.f, ah);
+        }
+        lo = al * s;
+        hi = ah * s;
+    } else if constexpr (WAV == 1 && QM == 2 && NB == 1) {
         float a, b;
         halves_to_float(w[0], a, b);
         lo = a * s;
@@ -324,7 +338,7 @@ __device__ __forceinline__ void sub_fetch(const TileArgs &a, const PlaneGeom &pg
 
 // Dequantised values of NW words into out[2 NW].
 template <int WAV, int NB, int QM, int NW>
-__device__ __forceinline__ void dq_row(const TileArgs &a, const uint32_t (&w)[NB][NW], float s,
+__device__ __forceinline__ void dq_row(const TileArgs &a, const uint32_t (&w)[NB][NW], float s, int plane,
                                        typename SV<WAV>::T (&out)[2 * NW]) {
     const int st = (int)a.g.step;
 #pragma unroll
@@ -332,7 +346,7 @@ __device__ __forceinline__ void dq_row(const TileArgs &a, const uint32_t (&w)[NB
         uint32_t x[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) x[b] = w[b][k];
-        dq_word<WAV, NB, QM>(x, a.bands, s, st, out[2 * k], out[2 * k + 1]);
+        dq_word<WAV, NB, QM>(x, a.bands, s, st, plane, out[2 * k], out[2 * k + 1]);
     }
 }
 
@@ -525,7 +539,7 @@ __device__ __forceinline__ uint32_t pack4_sat(int p0, int p1, int p2, int p3) {
 // right side (mirror_row, and codes loaded one at a time for the edge lanes
 // of planes narrower than 256).
 
-template <int WAV, int NB, int QM, bool EDGE, bool FOV = false>
+template <int WAV, int NB, int QM, bool EDGE, bool FOV = false, bool F32 = false>
 __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float *ring, uint32_t *stage,
                                            int lane) {
     using T = typename SV<WAV>::T;
@@ -651,11 +665,11 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
 #endif
                 }
                 sub_fetch<NB, 1, FOV>(a, pg, 2, 1, 1, W2, ke, l2, [&](int b) { return St::l2(sb, 1, b, lane); }, w);
-                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][1], hl);
+                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][1], plane, hl);
                 sub_fetch<NB, 1, FOV>(a, pg, 2, 2, 0, W2, ko, l2, [&](int b) { return St::l2(sb, 2, b, lane); }, w);
-                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][2], lh);
+                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][2], plane, lh);
                 sub_fetch<NB, 1, FOV>(a, pg, 2, 3, 1, W2, ko, l2, [&](int b) { return St::l2(sb, 3, b, lane); }, w);
-                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][3], hh);
+                dq_row<WAV, NB, QM, 1>(a, w, a.scale[2][3], plane, hh);
                 ev[0] = ll[0];
                 ev[1] = hl[0];
                 ev[2] = ll[1];
@@ -721,11 +735,11 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
                     }
                     uint32_t w[NB][2];
                     sub_fetch<NB, 2, FOV>(a, pg, 1, 1, 1, W, ke, l1, [&](int b) { return St::l1(sb, h, 1, b, lane); }, w);
-                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][1], hl);
+                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][1], plane, hl);
                     sub_fetch<NB, 2, FOV>(a, pg, 1, 2, 0, W, ko, l1, [&](int b) { return St::l1(sb, h, 2, b, lane); }, w);
-                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][2], lh);
+                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][2], plane, lh);
                     sub_fetch<NB, 2, FOV>(a, pg, 1, 3, 1, W, ko, l1, [&](int b) { return St::l1(sb, h, 3, b, lane); }, w);
-                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][3], hh);
+                    dq_row<WAV, NB, QM, 2>(a, w, a.scale[1][3], plane, hh);
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         ev[2 * m] = ll[m];
@@ -748,20 +762,37 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
                     for (int rr2 = 0; rr2 < 2; ++rr2) {
                         const T *v = rr2 ? oo : oe;
                         const size_t o = (size_t)(r0 + rr2) * W + l1.c0;
-                        int p[8];
-#pragma unroll
-                        for (int m = 0; m < 8; ++m) {
-                            if constexpr (WAV == 1) p[m] = __float2int_rd(v[m] + 128.5f);
-                            else p[m] = v[m] + 128;
-                        }
-                        // two groups of 4 samples: adjacent, or (chroma groups)
-                        // with the other chroma plane's group between them
+                        if constexpr (F32) {
 #if WV_CHECKED
-                        if (!checked_in((long long)o + 7, (long long)W * H, a.err)) continue;
+                            if (!checked_in((long long)o + 7, (long long)W * H, a.err)) continue;
 #endif
-                        uint32_t *d = reinterpret_cast<uint32_t *>(out8 + (o << pair_sh));
-                        d[0] = pack4_sat(p[0], p[1], p[2], p[3]);
-                        d[1 << pair_sh] = pack4_sat(p[4], p[5], p[6], p[7]);
+                            float *d = a.out_f32 + o;
+                            float f[8];
+#pragma unroll
+                            for (int m = 0; m < 8; ++m) f[m] = (float)v[m] + 128.0f;
+                            if ((reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+                                *reinterpret_cast<float4 *>(d) = make_float4(f[0], f[1], f[2], f[3]);
+                                *reinterpret_cast<float4 *>(d + 4) = make_float4(f[4], f[5], f[6], f[7]);
+                            } else {
+#pragma unroll
+                                for (int m = 0; m < 8; ++m) d[m] = f[m];
+                            }
+                        } else {
+                            int p[8];
+#pragma unroll
+                            for (int m = 0; m < 8; ++m) {
+                                if constexpr (WAV == 1) p[m] = __float2int_rd(v[m] + 128.5f);
+                                else p[m] = v[m] + 128;
+                            }
+                            // two groups of 4 samples: adjacent, or (chroma groups)
+                            // with the other chroma plane's group between them
+#if WV_CHECKED
+                            if (!checked_in((long long)o + 7, (long long)W * H, a.err)) continue;
+#endif
+                            uint32_t *d = reinterpret_cast<uint32_t *>(out8 + (o << pair_sh));
+                            d[0] = pack4_sat(p[0], p[1], p[2], p[3]);
+                            d[1 << pair_sh] = pack4_sat(p[4], p[5], p[6], p[7]);
+                        }
                     }
                 }
             }
@@ -770,55 +801,74 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
     }
 }
 
-template <int WAV, int NB, int QM>
-__global__ void __launch_bounds__(32 * kStripWarps, 3) k_strip(TileArgs a) {
-    __shared__ __align__(16) float rings[kStripWarps][kRing * kRingW];
-    extern __shared__ __align__(16) uint32_t stages[];   // kStripWarps x kStages x Stage<NB>::kWords
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    float *ring = rings[wi];
-    uint32_t *stage = stages + (size_t)wi * kStages * Stage<NB>::kWords;
+// One warp per CTA.  A launch has room for 12 strips per SM (168 registers a
+// thread) and lasts as long as its slowest tile, so warps that find no tile
+// or finish early must give their registers and shared memory back at once:
+// the coarse pass of the next viewport and the resampling of the previous one
+// run beside this kernel on what is free.  With four warps per CTA the slots
+// of a CTA stayed taken until its last warp was done: 8 viewports of an
+// 8192^2 stream 1049 -> 969 us, 4 of 6144 x 3072 218 -> 186 us.
+constexpr int kStripCtasPerSm = 12;
+
+template <int WAV, int NB, int QM, bool F32>
+__global__ void __launch_bounds__(32, kStripCtasPerSm) k_strip(TileArgs a, AllTiles all) {
+    __shared__ __align__(16) float ring[kRing * kRingW];
+    extern __shared__ __align__(16) uint32_t stage[];   // kStages x Stage<NB>::kWords
+    const int lane = threadIdx.x;
     for (int i = lane; i < kRing * kRingW; i += 32) ring[i] = 0.f;
     __syncwarp();
-    const int count = *(volatile const int *)a.count;
-    // tiles are dealt to the CTAs first and to their warps second, so every
-    // SM gets the same share of busy warps
-    for (int t = blockIdx.x + wi * gridDim.x; t < count; t += kStripWarps * gridDim.x) {
-        const uint32_t e = a.tiles[t];
+    int count = all.n;
+    if (count == 0) count = *(volatile const int *)a.count;
+    for (int t = blockIdx.x; t < count; t += gridDim.x) {
+        const uint32_t e = all.n ? all.entry(t) : a.tiles[t];
         if (strip_interior((int)(e & 0x3fff), a.g.p[(e >> 28) & 3].w))
-            strip_tile<WAV, NB, QM, false>(a, e, ring, stage, lane);
+            strip_tile<WAV, NB, QM, false, false, F32>(a, e, ring, stage, lane);
         else
-            strip_tile<WAV, NB, QM, true>(a, e, ring, stage, lane);
+            strip_tile<WAV, NB, QM, true, false, F32>(a, e, ring, stage, lane);
     }
 }
 
-template <int WAV, int NB, int QM>
-cudaError_t launch_s(const TileArgs &a, cudaStream_t cs) {
-    // stage memory is fixed per instantiation: opt in once per device
-    static std::once_flag once[64];
-    static cudaError_t set_err[64];
-    const int smem = kStripWarps * kStages * Stage<NB>::kWords * 4;
-    int dev = 0, sms = 148;
+// Grid of a strip kernel on the current device: its resident CTAs (stage
+// memory is fixed per instantiation: opted in and asked for once per device).
+struct StripGrid {
+    std::once_flag once;
+    cudaError_t err;
+    int ctas;
+};
+cudaError_t strip_grid(StripGrid *per_dev, const void *fn, int smem, int *ctas) {
+    int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::call_once(once[dev], [&] {
-        set_err[dev] = cudaFuncSetAttribute(k_strip<WAV, NB, QM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    StripGrid &G = per_dev[dev];
+    std::call_once(G.once, [&] {
+        int sms = 148, per_sm = 0;
+        G.err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (G.err == cudaSuccess) G.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (G.err == cudaSuccess) G.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32, smem);
+        G.ctas = sms * std::max(per_sm, 1);
     });
-    if (set_err[dev] != cudaSuccess) return set_err[dev];
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_strip<WAV, NB, QM>, 32 * kStripWarps, smem);
+    *ctas = G.ctas;
+    return G.err;
+}
+
+template <int WAV, int NB, int QM, bool F32>
+cudaError_t launch_s(const TileArgs &a, const AllTiles &all, cudaStream_t cs) {
+    static StripGrid per_dev[64];
+    constexpr int smem = kStages * Stage<NB>::kWords * 4;
+    int ctas = 0;
+    const cudaError_t e = strip_grid(per_dev, (const void *)k_strip<WAV, NB, QM, F32>, smem, &ctas);
     if (e != cudaSuccess) return e;
-    k_strip<WAV, NB, QM><<<sms * std::max(per_sm, 1), 32 * kStripWarps, smem, cs>>>(a);
+    k_strip<WAV, NB, QM, F32><<<all.n ? std::min(all.n, ctas) : ctas, 32, smem, cs>>>(a, all);
     return cudaGetLastError();
 }
 
-template <int WAV, int QM>
-cudaError_t launch_nb(const TileArgs &a, cudaStream_t cs) {
+template <int WAV, int QM, bool F32 = false>
+cudaError_t launch_nb(const TileArgs &a, const AllTiles &all, cudaStream_t cs) {
     switch (a.bands.n) {
-    case 1: return launch_s<WAV, 1, QM>(a, cs);
-    case 2: return launch_s<WAV, 2, QM>(a, cs);
-    case 3: return launch_s<WAV, 3, QM>(a, cs);
-    default: return launch_s<WAV, 4, QM>(a, cs);
+    case 1: return launch_s<WAV, 1, QM, F32>(a, all, cs);
+    case 2: return launch_s<WAV, 2, QM, F32>(a, all, cs);
+    case 3: return launch_s<WAV, 3, QM, F32>(a, all, cs);
+    default: return launch_s<WAV, 4, QM, F32>(a, all, cs);
     }
 }
 
@@ -827,17 +877,15 @@ cudaError_t launch_nb(const TileArgs &a, cudaStream_t cs) {
 // List entries are (surface, strip entry); a tile reads its surface's
 // arguments from the job table (read-only, through the cache).
 template <int WAV, int NB, int QM, bool FOV>
-__global__ void __launch_bounds__(32 * kStripWarps, 3)
+__global__ void __launch_bounds__(32, kStripCtasPerSm)
     k_strip_batch(const SurfaceJob *__restrict__ surfs, const uint2 *__restrict__ list, const int *count_p) {
-    __shared__ __align__(16) float rings[kStripWarps][kRing * kRingW];
-    extern __shared__ __align__(16) uint32_t stages[];   // kStripWarps x kStages x Stage<NB>::kWords
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-    float *ring = rings[wi];
-    uint32_t *stage = stages + (size_t)wi * kStages * Stage<NB>::kWords;
+    __shared__ __align__(16) float ring[kRing * kRingW];
+    extern __shared__ __align__(16) uint32_t stage[];   // kStages x Stage<NB>::kWords
+    const int lane = threadIdx.x;
     for (int i = lane; i < kRing * kRingW; i += 32) ring[i] = 0.f;
     __syncwarp();
     const int count = *(volatile const int *)count_p;
-    for (int t = blockIdx.x + wi * gridDim.x; t < count; t += kStripWarps * gridDim.x) {
+    for (int t = blockIdx.x; t < count; t += gridDim.x) {
         const uint2 it = list[t];
         const TileArgs &a = surfs[it.x].fine;
         const uint32_t e = it.y;
@@ -850,23 +898,12 @@ __global__ void __launch_bounds__(32 * kStripWarps, 3)
 
 template <int WAV, int NB, int QM, bool FOV>
 cudaError_t launch_b(const SurfaceJob *surfs, const uint2 *list, const int *count, cudaStream_t cs) {
-    static std::once_flag once[64];
-    static cudaError_t set_err[64];
-    const int smem = kStripWarps * kStages * Stage<NB>::kWords * 4;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::call_once(once[dev], [&] {
-        set_err[dev] =
-            cudaFuncSetAttribute(k_strip_batch<WAV, NB, QM, FOV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    });
-    if (set_err[dev] != cudaSuccess) return set_err[dev];
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_strip_batch<WAV, NB, QM, FOV>,
-                                                                  32 * kStripWarps, smem);
+    static StripGrid per_dev[64];
+    constexpr int smem = kStages * Stage<NB>::kWords * 4;
+    int ctas = 0;
+    const cudaError_t e = strip_grid(per_dev, (const void *)k_strip_batch<WAV, NB, QM, FOV>, smem, &ctas);
     if (e != cudaSuccess) return e;
-    k_strip_batch<WAV, NB, QM, FOV><<<sms * std::max(per_sm, 1), 32 * kStripWarps, smem, cs>>>(surfs, list, count);
+    k_strip_batch<WAV, NB, QM, FOV><<<ctas, 32, smem, cs>>>(surfs, list, count);
     return cudaGetLastError();
 }
 
@@ -889,13 +926,20 @@ cudaError_t launch_decode_strips_batch(int wavelet, int nb, bool fovea, bool dz_
     return fovea ? launch_b<0, 2, 0, true>(surfs, list, count, cs) : launch_b<0, 2, 0, false>(surfs, list, count, cs);
 }
 
-// Levels 2 and 1 of the listed strip tiles, LL_2 from the planes written by
-// the coarse pass (streams of three or more levels).
+// Float samples come from kernels of their own (the store path in the 8-bit
+// kernels cost them 16 spilled bytes and 9 % of their time), for the code
+// forms every stream has but the rare ones (9/7 with |q| > kDzTMax: square
+// tiles).
+bool strip_float_supported(const Geom &g) { return g.quant == 0 && (g.wavelet == WV_WAVELET_53 || g.dz_t); }
+
+// Levels 2 and 1 of the listed strip tiles (all_plane >= 0: of every strip of
+// that plane, no list), LL_2 from the planes written by the coarse pass
+// (streams of three or more levels).
 cudaError_t launch_decode_strips(const Geom &g, const int16_t *payload, const int32_t *table,
                                  const Bands &bands, const float *const *ll2, const int *ll2_pitch,
                                  uint8_t *const *out_u8, float *out_f32, int f32_plane,
                                  const uint32_t *tiles, int *counters, int *err, cudaStream_t cs,
-                                 bool chroma_pairs) {
+                                 bool chroma_pairs, int all_plane) {
     if (chroma_pairs && (g.planes != 3 || out_u8[2] != out_u8[1] + 4 || ((uintptr_t)out_u8[1] & 15)))
         return cudaErrorInvalidValue;
     TileArgs a;
@@ -914,18 +958,38 @@ cudaError_t launch_decode_strips(const Geom &g, const int16_t *payload, const in
         a.ll_in_pitch[p] = ll2 ? ll2_pitch[p] : 0;
         a.out_u8[p] = out_u8[p];
     }
-    // 8-bit samples only (float output takes the square-tile pass): the
-    // float store path cost the kernel 16 spilled bytes and 9 % of its time
-    if (out_f32) return cudaErrorInvalidValue;
-    (void)f32_plane;
+    if (out_f32 && (all_plane < 0 || f32_plane != all_plane || !strip_float_supported(g))) return cudaErrorInvalidValue;
+    a.out_f32 = out_f32;
+    a.f32_plane = out_f32 ? f32_plane : -1;
     a.out_pair = chroma_pairs ? 1 : 0;
     a.tiles = tiles;
     a.count = counters;
-    a.work = counters + 2;
     fill_tile_scales(a);
-    if (!g.strip || g.levels < 3 || g.quant != 0 || !ll2) return cudaErrorInvalidValue;
-    if (g.wavelet == WV_WAVELET_97) return g.dz_t ? launch_nb<1, 2>(a, cs) : launch_nb<1, 0>(a, cs);
-    return launch_nb<0, 0>(a, cs);
+    if (!g.strip || g.levels < 3 || !ll2) return cudaErrorInvalidValue;
+    AllTiles all{};
+    if (all_plane >= 0) {
+        // Every strip of one plane, in any height: the lowest that leaves an
+        // SM at most half of its 12 warp slots (the launch lasts one tile; a
+        // tile of h rows takes h / 4 + 7 iterations, and twice the warps on
+        // an SM do not double an iteration's time), else the default.  The
+        // planes of a 2048 x 1024 4:2:0 frame: 64 rows, with tile lists 255
+        // us; this 138, with coarse tiles of 32 115.
+        const PlaneGeom &pg = g.p[all_plane];
+        int dev = 0, sms = 148;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        a.th = kStripH;
+        for (int h = 16; h < kStripH; h *= 2)
+            if (pg.tiles_x * ((pg.h + h - 1) / h) <= kStripCtasPerSm / 2 * sms) {
+                a.th = h;
+                break;
+            }
+        all = AllTiles{pg.tiles_x * ((pg.h + a.th - 1) / a.th), all_plane, pg.tiles_x};
+    }
+    if (out_f32) return g.wavelet == WV_WAVELET_97 ? launch_nb<1, 2, true>(a, all, cs) : launch_nb<0, 0, true>(a, all, cs);
+    if (g.quant == 1) return g.wavelet == WV_WAVELET_97 ? launch_nb<1, 1>(a, all, cs) : cudaErrorInvalidValue;
+    if (g.wavelet == WV_WAVELET_97) return g.dz_t ? launch_nb<1, 2>(a, all, cs) : launch_nb<1, 0>(a, all, cs);
+    return launch_nb<0, 0>(a, all, cs);
 }
 
 }  // namespace wv

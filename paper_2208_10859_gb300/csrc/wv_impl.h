@@ -69,6 +69,7 @@ struct Geom {
     int total_ctiles;
     int tw, th;  // output tile width and height (plane pixels): square 64 or 128, or a strip kStripW x th
     int strip;   // 1: output tiles are strips decoded by the strip kernel (strip.cu)
+    int halves;  // 1: every strip is listed as two half strips (0: edge strips only)
     int ctile;   // coarse tile side (LL_2 samples): 32 or 64
     // LL_2 window an output tile (tx, ty) reads: columns (tw / 4) tx + wx0 ..
     // (tw / 4) tx + wx1, rows (th / 4) ty + wy0 .. (th / 4) ty + wy1 (before
@@ -149,7 +150,6 @@ struct TileArgs {
     const uint8_t *fmask;    // foveation bits per mask cell (bit l-1: keep level l), or null
     const uint32_t *tiles;   // tile list (count entries)
     const int *count;
-    int *work;               // strip kernel: next tile to take (zeroed before the launch)
     int *err;
     // payload blocks held (0: not checked; streams validate their table when
     // opened): a table entry at or above it reads as an absent block and
@@ -169,6 +169,19 @@ struct TileArgs {
     // samples.  (The half: the midpoint reconstruction is computed as
     // (2q + sign q) step / 2.)
     float scale[kMaxLevels + 1][4];
+};
+
+// Every tile of one plane instead of a list (n > 0: n tiles, nx per row).  A
+// kernel argument of its own: a kernel that chooses between a field of a
+// struct argument and a value in memory may read the wrong one's address
+// space, or keeps a copy of the struct in local memory.
+struct AllTiles {
+    int n, plane, nx;
+#ifdef __CUDACC__
+    __device__ __forceinline__ uint32_t entry(int t) const {
+        return ((uint32_t)plane << 28) | ((uint32_t)(t / nx) << 14) | (uint32_t)(t % nx);
+    }
+#endif
 };
 
 // Bilinear reprojection of one viewport from decoded planes.
@@ -263,6 +276,20 @@ int build_geom_rect(const wv_stream_desc &d, Geom *g, int tw, int th, int ctile)
 // for streams the strip kernel decodes (strip_eligible), else WV_ERR_ARG.
 int build_geom_strip(const wv_stream_desc &d, Geom *g, int th = kStripH, int ctile = kCoarseTile);
 bool strip_eligible(const wv_stream_desc &d, uint64_t n_payload);
+// Strips of 64 rows of a frame (of one eye's part) up to which its streams are
+// cut finer: strips of 32 rows and coarse tiles of 32 LL_2 samples, and up to
+// a quarter of that every strip listed as two halves.  A viewport shows about
+// a quarter of the frame, and a launch lasts as long as its slowest tile (a
+// strip of h rows takes h / 4 + 7 iterations of one warp), so while a
+// viewport's tiles do not fill the chip, lower tiles finish sooner; they redo
+// more warm-up rows, which costs once the chip is full.  The line is where a
+// viewport's 32-row strips are eight warps per SM (152 SMs).  Default against
+// finer tiles: 4 viewports of 2880 x 1440 229 -> 145 us, of 4096 x 2048 per eye
+// 272 -> 214 us, of 6144 x 3072 186 -> 174 us; 8 of 8192^2 (above the line)
+// 961 -> 1031 us.  Halves everywhere below the line: 6144 x 3072 174 -> 186 us.
+constexpr int kFineStrips = 16 * 152;
+int viewable_strips(const wv_stream_desc &d);   // 64-row strips of what an eye can see
+
 Bands frame_bands(const Geom &g, int frame);
 View make_view(float yaw, float pitch, float fov, int out_w, int out_h, int eq_w, int eq_h, int row0 = 0);
 int eye_view(const Geom &g, int eye, int *row0, int *rows);   // WV_ERR_ARG for an invalid eye
@@ -286,12 +313,14 @@ cudaError_t launch_decode_tiles(const Geom &g, const int16_t *payload, const int
                                 int *err, cudaStream_t cs, int n_slots = 0);
 cudaError_t launch_decode_coarse(const Geom &g, const int16_t *payload, const int32_t *table,
                                  const Bands &bands, float *const *ll2, const int *ll2_pitch,
-                                 const uint32_t *tiles, const int *count, int *err, cudaStream_t cs);
+                                 const uint32_t *tiles, const int *count, int *err, cudaStream_t cs,
+                                 int all_plane = -1);
 cudaError_t launch_decode_strips(const Geom &g, const int16_t *payload, const int32_t *table,
                                  const Bands &bands, const float *const *ll2, const int *ll2_pitch,
                                  uint8_t *const *out_u8, float *out_f32, int f32_plane,
                                  const uint32_t *tiles, int *counters, int *err, cudaStream_t cs,
-                                 bool chroma_pairs = false);
+                                 bool chroma_pairs = false, int all_plane = -1);
+bool strip_float_supported(const Geom &g);
 // Batched strip fine pass: the strip tiles (list of (surface, entry)) of the
 // decode targets of one class whose coarse tiles are done; classes with up
 // to two coefficient frames, 9/7 codes held as 2q + sign(q) or 5/3.
