@@ -106,6 +106,8 @@ struct wv_batch {
     int device = 0;
     cudaStream_t cs = nullptr;         // stream of the last launch
     cudaStream_t cap = nullptr;        // private stream for graph capture
+    std::vector<cudaStream_t> side;    // further ones, for the branches of a captured graph
+    cudaEvent_t fork = nullptr, join = nullptr;
     char *dmem = nullptr;
     size_t dbytes = 0;
     char *host = nullptr;              // pinned job-table staging
@@ -177,6 +179,11 @@ int plan_batch(const wv_batch *b, const wv_request *reqs, int n, Plan &P) {
     P.surf.clear();
     P.waves.clear();
     P.req_surface.assign(n, -1);
+    // a small batch is cut as finely as a small stream (kFineStrips; there a
+    // viewport's share of the frame, here the sum over the requests)
+    long long strips = 0;
+    for (int i = 0; i < n; ++i) strips += viewable_strips(reqs[i].s->desc);
+    const bool fine = strips <= kFineStrips;
     for (int i = 0; i < n; ++i) {
         const wv_request &r = reqs[i];
         if (!r.fovea && b->share) {
@@ -196,9 +203,11 @@ int plan_batch(const wv_batch *b, const wv_request *reqs, int n, Plan &P) {
         // the class (the tuned square shape then only sets the coarse tile)
         S.strip = b->strips && strip_eligible(r.s->desc, r.s->n_payload) &&
                   strip_batch_supported(sg.wavelet, 1 + sg.tlevels, sg.dz_t);
-        const int gr = S.strip ? build_geom_strip(r.s->desc, &S.g, kStripH, ts.ctile)
+        const bool tuned = b->tuned.count(TuneKey{sg.wavelet, sg.levels, sg.p[0].w, sg.p[0].h}) != 0;
+        const int gr = S.strip ? build_geom_strip(r.s->desc, &S.g, fine ? 32 : kStripH, fine && !tuned ? 32 : ts.ctile)
                                : build_geom_rect(r.s->desc, &S.g, ts.tw, ts.th, ts.ctile);
         if (gr != WV_OK) return WV_ERR_ARG;
+        S.g.halves = S.strip && strips <= kFineStrips / 4;
         S.g.dz_t = sg.dz_t;   // the code form of the stream's device payload
         S.g.n_blocks = sg.n_blocks;
         // 1 + tlevels coefficient frames
@@ -405,6 +414,33 @@ void fill_jobs(wv_batch *b, const wv_request *reqs, int n, Plan &P) {
     }
 }
 
+// One decode class of a wave: its coarse tiles and square fine tiles, then its
+// strip tiles.
+cudaError_t launch_class(wv_batch *b, const Plan &P, const Wave &W, int c, const BatchLists &lists, cudaStream_t cs) {
+    const SurfaceJob *surfs = (const SurfaceJob *)(b->dmem + P.jobs) + W.s0;
+    int *ctr = (int *)(b->dmem + W.ctr);
+    const int group = c / kMaxBands, wavelet = group >= 4 ? WV_WAVELET_97 : group / 2;
+    const cudaError_t e = launch_decode_batch(wavelet, c % kMaxBands + 1, group % 2 == 1, group >= 4, surfs,
+                                              lists.coarse[c], lists.fine[c], ctr + 4 * c, ctr + kBatchCtr,
+                                              (int *)(b->dmem + P.err), (const int *)(b->dmem + kWaitWord),
+                                              W.smem[c], cs);
+    if (e != cudaSuccess || !W.strip[c]) return e;
+    return launch_decode_strips_batch(wavelet, c % kMaxBands + 1, group % 2 == 1, group >= 4, surfs, lists.strip[c],
+                                      ctr + 4 * c + 3, cs);
+}
+
+// Streams and events for up to n branches (a graph of one branch without them).
+void ensure_branches(wv_batch *b, size_t n) {
+    if (!b->fork && cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess) b->fork = nullptr;
+    if (!b->join && cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess) b->join = nullptr;
+    while (b->fork && b->join && b->side.size() + 1 < n) {
+        cudaStream_t st = nullptr;
+        if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) break;
+        b->side.push_back(st);
+    }
+    cudaGetLastError();
+}
+
 // Enqueue the batch on cs (captured into a graph, or run directly with
 // events between the steps when timed).
 cudaError_t enqueue(wv_batch *b, const Plan &P, int n, cudaStream_t cs, bool timed) {
@@ -438,23 +474,22 @@ cudaError_t enqueue(wv_batch *b, const Plan &P, int n, cudaStream_t cs, bool tim
         }
         launch_select_batch(surfs + W.s0, m, W.max_stamps, lists, ctr, cs);
         if (timed) cudaEventRecord(ev[2], cs);
-        for (int c = 0; c < kClasses; ++c) {
-            if (!W.smem[c]) continue;
-            const int group = c / kMaxBands;
-            e = launch_decode_batch(group >= 4 ? WV_WAVELET_97 : group / 2, c % kMaxBands + 1, group % 2 == 1,
-                                    group >= 4, surfs + W.s0, lists.coarse[c], lists.fine[c], ctr + 4 * c,
-                                    ctr + kBatchCtr, (int *)(base + P.err), (const int *)(base + kWaitWord),
-                                    W.smem[c], cs);
-            if (e != cudaSuccess) return e;
+        // The classes are independent until the resampling: each is a branch of
+        // the captured graph (coarse tiles, then its strip tiles), so the tail
+        // of one class's launch overlaps the others' work.
+        std::vector<int> classes;
+        for (int c = 0; c < kClasses; ++c)
+            if (W.smem[c]) classes.push_back(c);
+        const bool branch = cs == b->cap && classes.size() > 1 && b->side.size() + 1 >= classes.size();
+        if (branch) e = cudaEventRecord(b->fork, cs);
+        for (size_t k = 0; k < classes.size() && e == cudaSuccess; ++k) {
+            const cudaStream_t bs = branch && k > 0 ? b->side[k - 1] : cs;
+            if (bs != cs) e = cudaStreamWaitEvent(bs, b->fork, 0);
+            if (e == cudaSuccess) e = launch_class(b, P, W, classes[k], lists, bs);
+            if (bs != cs && e == cudaSuccess) e = cudaEventRecord(b->join, bs);
+            if (bs != cs && e == cudaSuccess) e = cudaStreamWaitEvent(cs, b->join, 0);
         }
-        // the strip tiles, once their class's coarse tiles are done
-        for (int c = 0; c < kClasses; ++c) {
-            if (!W.strip[c]) continue;
-            const int group = c / kMaxBands;
-            e = launch_decode_strips_batch(group >= 4 ? WV_WAVELET_97 : group / 2, c % kMaxBands + 1, group % 2 == 1,
-                                           group >= 4, surfs + W.s0, lists.strip[c], ctr + 4 * c + 3, cs);
-            if (e != cudaSuccess) return e;
-        }
+        if (e != cudaSuccess) return e;
         if (timed) cudaEventRecord(ev[3], cs);
         launch_resample_batch(rq + W.r0, nr, W.max_w, W.max_h, cs);
         if (timed) cudaEventRecord(ev[4], cs);
@@ -558,6 +593,10 @@ int run_batch(wv_batch *b, const wv_request *reqs, int n, cudaStream_t cs) {
             if (b->exec) cudaGraphExecDestroy(b->exec);
             b->exec = nullptr;
             cudaGraph_t graph = nullptr;
+            size_t branches = 0;
+            for (const Wave &W : P.waves)
+                branches = std::max(branches, (size_t)std::count_if(W.smem, W.smem + kClasses, [](int m) { return m != 0; }));
+            ensure_branches(b, branches);
             e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeRelaxed);
             if (e == cudaSuccess) {
                 const cudaError_t e1 = enqueue(b, P, n, b->cap, false);
@@ -637,6 +676,9 @@ void wv_batch_close(wv_batch *b) {
     for (cudaEvent_t e : b->ev)
         if (e) cudaEventDestroy(e);
     if (b->cap) cudaStreamDestroy(b->cap);
+    for (cudaStream_t st : b->side) cudaStreamDestroy(st);
+    for (cudaEvent_t e : {b->fork, b->join})
+        if (e) cudaEventDestroy(e);
     delete b;
 }
 
