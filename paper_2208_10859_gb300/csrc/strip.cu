@@ -101,6 +101,7 @@ __device__ __forceinline__ void dq_word(const uint32_t (&w)[NB], const Bands &bd
         float al = 0.f, ah = 0.f;
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
+            if (w[b] == 0u) continue;   // most words of a record stream; they add 0
             const float c0 = bd.qp[b][plane][1][0], d = bd.qp[b][plane][1][1];
             const float sg = (b == 0 || bd.bit[b]) ? 1.f : -1.f;
             const int ql = lo16(w[b]), qh = hi16(w[b]);
@@ -580,11 +581,6 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
     const int pair_sh = a.out_pair && plane > 0 ? 1 : 0;
 
     SubRow<NB> r2[4], r1[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        r2[k].by = -1;
-        r1[k].by = -1;
-    }
     VCols<WAV, 4> v2;
     VCols<WAV, 8> v1;
     v2.clear();
@@ -628,6 +624,19 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
         }
         cp_commit();
     };
+    // the first rows' table entries, all in flight at once (the copies of a
+    // subband wait for its entries)
+    {
+        const int lb = g.log2b, s2 = (Y0 >> 1) - 6, s1 = Y0 - 4;
+        const int ke2 = refl(s2, H2) >> 1, ko2 = refl(s2 + 1, H2) >> 1;
+        const int ke1 = refl(s1, H) >> 1, ko1 = refl(s1 + 1, H) >> 1;
+        sub_refresh<NB>(a, pg, 2, 1, ke2 >> lb, l2, r2[1]);
+        sub_refresh<NB>(a, pg, 2, 2, ko2 >> lb, l2, r2[2]);
+        sub_refresh<NB>(a, pg, 2, 3, ko2 >> lb, l2, r2[3]);
+        sub_refresh<NB>(a, pg, 1, 1, ke1 >> lb, l1, r1[1]);
+        sub_refresh<NB>(a, pg, 1, 2, ko1 >> lb, l1, r1[2]);
+        sub_refresh<NB>(a, pg, 1, 3, ko1 >> lb, l1, r1[3]);
+    }
 #pragma unroll 1
     for (int t = 0; t < kStages - 1; ++t) {
         if (t < NT) issue(t);
