@@ -117,8 +117,11 @@ int stream_geoms(const wv_stream_desc &d, uint64_t n_payload, Geom *g, Geom *gsq
 }
 
 struct Layout {
-    size_t payload, table, recon[3], ll2[3], mask, tiles, ctiles, tile_gen, ctile_gen, counters, err;
-    size_t ll2_1[3], tiles1, ctiles1, counters1, recon1[3], total;   // the second per-viewport set
+    size_t payload, table, mask, err, total;
+    int n_sets;
+    struct Set {
+        size_t recon[3], ll2[3], tiles, ctiles, tile_gen, ctile_gen, counters, end;
+    } set[kViewSets];   // the buffers of the viewports in flight
 };
 
 // Device layout of a stream; tile lists and stamps hold the larger tile count
@@ -134,43 +137,34 @@ Layout layout(const Geom &g0, const Geom &gsq, uint64_t n_payload) {
     o = align256(o + n_payload * g.block * g.block * 2);
     L.table = o;
     o = align256(o + (size_t)g.num_frames * g.nbpf * 4);
-    for (int p = 0; p < 3; ++p) {
-        L.recon[p] = o;
-        if (p < g.planes) o = align256(o + (size_t)g.p[p].w * g.p[p].h);
-    }
-    for (int p = 0; p < 3; ++p) {
-        L.ll2[p] = o;
-        if (p < g.planes && g.levels >= 3)
-            o = align256(o + (size_t)g.p[p].ll2_pitch * (g.p[p].h >> 2) * 4);
-    }
     L.mask = o;
     o = align256(o + (size_t)g.cells_x * g.cells_y);
-    L.tiles = o;
-    o = align256(o + list_tiles * 4);
-    L.ctiles = o;
-    o = align256(o + (size_t)(g.total_ctiles > 0 ? g.total_ctiles : 1) * 4);
-    L.tile_gen = o;
-    o = align256(o + (size_t)g.total_tiles * 4);
-    L.ctile_gen = o;
-    o = align256(o + (size_t)(g.total_ctiles > 0 ? g.total_ctiles : 1) * 4);
-    L.counters = o;
-    o = align256(o + 64);
     L.err = o;
     o = align256(o + 64);
-    for (int p = 0; p < 3; ++p) {
-        L.ll2_1[p] = o;
-        if (p < g.planes && g.levels >= 3)
-            o = align256(o + (size_t)g.p[p].ll2_pitch * (g.p[p].h >> 2) * 4);
-    }
-    L.tiles1 = o;
-    o = align256(o + list_tiles * 4);
-    L.ctiles1 = o;
-    o = align256(o + (size_t)(g.total_ctiles > 0 ? g.total_ctiles : 1) * 4);
-    L.counters1 = o;
-    o = align256(o + 64);
-    for (int p = 0; p < 3; ++p) {
-        L.recon1[p] = o;
-        if (p < g.planes) o = align256(o + (size_t)g.p[p].w * g.p[p].h);
+    // one viewport at a time without a coarse pass (decode_region)
+    L.n_sets = g.levels < 3 ? 1 : g.strip && g.th == 32 ? kViewSets : kViewSetsLarge;
+    for (int k = 0; k < L.n_sets; ++k) {
+        Layout::Set &S = L.set[k];
+        for (int p = 0; p < 3; ++p) {
+            S.recon[p] = o;
+            if (p < g.planes) o = align256(o + (size_t)g.p[p].w * g.p[p].h);
+        }
+        for (int p = 0; p < 3; ++p) {
+            S.ll2[p] = o;
+            if (p < g.planes && g.levels >= 3)
+                o = align256(o + (size_t)g.p[p].ll2_pitch * (g.p[p].h >> 2) * 4);
+        }
+        S.tiles = o;
+        o = align256(o + list_tiles * 4);
+        S.ctiles = o;
+        o = align256(o + (size_t)(g.total_ctiles > 0 ? g.total_ctiles : 1) * 4);
+        S.tile_gen = o;
+        o = align256(o + (size_t)g.total_tiles * 4);
+        S.ctile_gen = o;
+        o = align256(o + (size_t)(g.total_ctiles > 0 ? g.total_ctiles : 1) * 4);
+        S.counters = o;
+        o = align256(o + 64);
+        S.end = o;
     }
     L.total = o;
     return L;
@@ -218,8 +212,9 @@ cudaError_t launch_fine(wv_stream *s, const Bands &b, const float *const *ll2, u
     const Geom &g = active_geom(s);
     if (strip_mode(s)) {
         // into the stream's reconstruction planes: chroma in alternating Cb, Cr groups
-        const bool own = (out_u8[1] == s->recon[1] && out_u8[2] == s->recon[2]) ||
-                         (out_u8[1] == s->recon1[1] && out_u8[2] == s->recon1[2]);
+        bool own = false;
+        for (int k = 0; k < s->n_sets; ++k)
+            own = own || (out_u8[1] == s->set[k].recon[1] && out_u8[2] == s->set[k].recon[2]);
         const bool pairs = own && recon_pairs(s);
         uint8_t *const outs[3] = {out_u8[0], out_u8[1], pairs ? out_u8[1] + 4 : out_u8[2]};
         return launch_decode_strips(g, s->payload, s->table, b, ll2, s->ll2_pitch, outs, f32, f32_plane, tiles,
@@ -232,21 +227,22 @@ cudaError_t launch_fine(wv_stream *s, const Bands &b, const float *const *ll2, u
 cudaError_t run_decode(wv_stream *s, const Bands &b, uint8_t *const *out_u8, float *f32,
                        int f32_plane, int all_plane = -1) {
     const Geom &g = active_geom(s);
+    const ViewSet &S = s->set[0];
     cudaError_t e;
     if (split_mode(s)) {
         prof_begin(s, kKCoarse);
-        e = launch_decode_coarse(g, s->payload, s->table, b, s->ll2, s->ll2_pitch, s->ctiles,
-                                 s->counters + 1, s->err, s->cs, all_plane);
+        e = launch_decode_coarse(g, s->payload, s->table, b, S.ll2, s->ll2_pitch, S.ctiles,
+                                 S.counters + 1, s->err, s->cs, all_plane);
         prof_end(s);
         if (e != cudaSuccess) return e;
-        const float *ll2c[3] = {s->ll2[0], s->ll2[1], s->ll2[2]};
+        const float *ll2c[3] = {S.ll2[0], S.ll2[1], S.ll2[2]};
         prof_begin(s, kKFine);
-        e = launch_fine(s, b, ll2c, out_u8, f32, f32_plane, s->tiles, s->counters, s->cs, all_plane);
+        e = launch_fine(s, b, ll2c, out_u8, f32, f32_plane, S.tiles, S.counters, s->cs, all_plane);
         prof_end(s);
         return e;
     }
     prof_begin(s, kKFine);
-    e = launch_decode_tiles(g, s->payload, s->table, b, out_u8, f32, f32_plane, s->tiles, s->counters, s->err,
+    e = launch_decode_tiles(g, s->payload, s->table, b, out_u8, f32, f32_plane, S.tiles, S.counters, s->err,
                             s->cs);
     prof_end(s);
     return e;
@@ -266,20 +262,18 @@ int eye_view(const Geom &g, int eye, int *row0, int *rows) {
     return WV_OK;
 }
 
-// The internal stream and events of the overlapped viewport path (created on
-// first use; the stream has the highest priority so that its small kernels
-// take SMs as soon as the running fine pass or resampling frees them).
-cudaError_t ensure_aux(wv_stream *s) {
-    if (s->aux) return cudaSuccess;
-    int lo = 0, hi = 0;
-    cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&s->aux, cudaStreamNonBlocking, hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->fs, cudaStreamNonBlocking);
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-        e = cudaEventCreateWithFlags(&s->ev_ready[k], cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_fine[k], cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_free[k], cudaEventDisableTiming);
-    }
+// The internal stream and events of set k (created when it is first used).
+// The set's first chain waits for everything enqueued on cs so far: work on
+// cs uses set 0.
+cudaError_t ensure_set(wv_stream *s, int k) {
+    ViewSet &S = s->set[k];
+    if (S.st) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (!S.fine) e = cudaEventCreateWithFlags(&S.fine, cudaEventDisableTiming);
+    if (e == cudaSuccess && !S.free) e = cudaEventCreateWithFlags(&S.free, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(S.free, s->cs);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking);
+    if (e != cudaSuccess) cudaGetLastError();
     return e;
 }
 
@@ -294,43 +288,33 @@ void check_capture(wv_stream *s) {
     }
 }
 
-// After work on cs that used the per-viewport buffers of set 0 (or both):
-// later overlapped viewports wait for it before reusing either set.
+// After work on cs that used the per-viewport buffers of set 0: later
+// overlapped viewports wait for it before reusing any set.
 void mark_sets_used(wv_stream *s) {
     check_capture(s);
-    if (!s->aux || !s->overlap) return;
-    cudaEventRecord(s->ev_free[0], s->cs);
-    cudaEventRecord(s->ev_free[1], s->cs);
+    if (!s->overlap) return;
+    for (int k = 0; k < s->n_sets; ++k)
+        if (s->set[k].st) cudaEventRecord(s->set[k].free, s->cs);
 }
 
-// Overlapped viewport decode into buffer set k, three stages on three
-// streams: footprint, selection and coarse pass on aux (once the fine pass
-// of two viewports ago and every cs use of set k are done), the fine pass
-// into set k's reconstruction on fs (once the coarse pass is done and the
-// resampling of two viewports ago has read that reconstruction), and cs
-// waits for the fine pass; the caller's resampling then runs on cs while
-// the next viewport's fine pass writes the other set.
+// Overlapped viewport decode into buffer set k: the whole chain on the set's
+// stream, once the resampling of the set's previous viewport has read its
+// reconstruction; cs waits for the chain, and the caller's resampling then
+// runs on cs beside the next viewports' chains.
 int decode_region_overlapped(wv_stream *s, const View &v, const Bands &b, uint32_t gen) {
     const Geom &g = active_geom(s);
     const int k = s->slot;
-    s->slot ^= 1;
-    uint32_t *tiles = k ? s->tiles1 : s->tiles, *ctiles = k ? s->ctiles1 : s->ctiles;
-    int *counters = k ? s->counters1 : s->counters;
-    float *ll2[3] = {k ? s->ll2_1[0] : s->ll2[0], k ? s->ll2_1[1] : s->ll2[1], k ? s->ll2_1[2] : s->ll2[2]};
-    uint8_t *const *recon = k ? s->recon1 : s->recon;
-    cudaError_t e = cudaStreamWaitEvent(s->aux, s->ev_fine[k], 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->aux, s->ev_free[k], 0);
+    s->slot = (k + 1) % s->n_sets;
+    ViewSet &S = s->set[k];
+    cudaError_t e = cudaStreamWaitEvent(S.st, S.free, 0);
     if (e != cudaSuccess) return WV_ERR_CUDA;
-    launch_footprint(g, v, s->mask, s->tile_gen, s->ctile_gen, gen, counters, s->aux);
-    launch_select_tiles(g, s->tile_gen, s->ctile_gen, gen, tiles, ctiles, counters, s->aux);
-    e = launch_decode_coarse(g, s->payload, s->table, b, ll2, s->ll2_pitch, ctiles, counters + 1, s->err, s->aux);
-    if (e == cudaSuccess) e = cudaEventRecord(s->ev_ready[k], s->aux);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->fs, s->ev_ready[k], 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->fs, s->ev_free[k], 0);
-    const float *ll2c[3] = {ll2[0], ll2[1], ll2[2]};
-    if (e == cudaSuccess) e = launch_fine(s, b, ll2c, recon, nullptr, -1, tiles, counters, s->fs);
-    if (e == cudaSuccess) e = cudaEventRecord(s->ev_fine[k], s->fs);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cs, s->ev_fine[k], 0);
+    launch_footprint(g, v, nullptr, S.tile_gen, S.ctile_gen, gen, S.counters, S.st);
+    launch_select_tiles(g, S.tile_gen, S.ctile_gen, gen, S.tiles, S.ctiles, S.counters, S.st);
+    e = launch_decode_coarse(g, s->payload, s->table, b, S.ll2, s->ll2_pitch, S.ctiles, S.counters + 1, s->err, S.st);
+    const float *ll2c[3] = {S.ll2[0], S.ll2[1], S.ll2[2]};
+    if (e == cudaSuccess) e = launch_fine(s, b, ll2c, S.recon, nullptr, -1, S.tiles, S.counters, S.st);
+    if (e == cudaSuccess) e = cudaEventRecord(S.fine, S.st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cs, S.fine, 0);
     s->cur = k;
     s->pending = true;
     return e == cudaSuccess ? WV_OK : WV_ERR_CUDA;
@@ -344,27 +328,28 @@ int decode_region(wv_stream *s, int frame, float yaw, float pitch, float fov, in
     const Bands b = stream_bands(s, frame);
     const uint32_t gen = next_gen(s);
     check_capture(s);
-    if (split_mode(s) && !s->prof && s->overlap && ensure_aux(s) == cudaSuccess)
+    if (split_mode(s) && !s->prof && s->overlap && ensure_set(s, s->slot) == cudaSuccess)
         return decode_region_overlapped(s, v, b, gen);
     prof_begin(s, kKFootprint);
-    launch_footprint(g, v, s->mask, s->tile_gen, s->ctile_gen, gen, s->counters, s->cs);
+    ViewSet &S = s->set[0];
+    launch_footprint(g, v, s->mask, S.tile_gen, S.ctile_gen, gen, S.counters, s->cs);
     prof_end(s);
     prof_begin(s, kKTiles);
-    launch_select_tiles(g, s->tile_gen, s->ctile_gen, gen, s->tiles, s->ctiles, s->counters, s->cs);
+    launch_select_tiles(g, S.tile_gen, S.ctile_gen, gen, S.tiles, S.ctiles, S.counters, s->cs);
     prof_end(s);
-    const cudaError_t e = run_decode(s, b, s->recon, nullptr, -1);
+    const cudaError_t e = run_decode(s, b, S.recon, nullptr, -1);
     mark_sets_used(s);
     s->cur = 0;
     s->pending = true;
     return e == cudaSuccess ? WV_OK : WV_ERR_CUDA;
 }
 
-uint8_t *const *recon_planes(const wv_stream *s) { return s->cur ? s->recon1 : s->recon; }
+uint8_t *const *recon_planes(const wv_stream *s) { return s->set[s->cur].recon; }
 
 void release_recon(wv_stream *s, bool again) {
     if (!s->pending && !again) return;
     s->pending = false;
-    if (s->aux && s->overlap) cudaEventRecord(s->ev_free[s->cur], s->cs);
+    if (s->set[s->cur].st && s->overlap) cudaEventRecord(s->set[s->cur].free, s->cs);
 }
 
 }  // namespace wv
@@ -838,26 +823,26 @@ int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t devi
     char *base = (char *)s->dmem;
     if (!host_payload) s->payload = (int16_t *)(base + L.payload);
     s->table = (int32_t *)(base + L.table);
-    for (int p = 0; p < 3; ++p) s->recon[p] = p < s->g.planes ? (uint8_t *)(base + L.recon[p]) : nullptr;
-    for (int p = 0; p < 3; ++p) s->recon1[p] = p < s->g.planes ? (uint8_t *)(base + L.recon1[p]) : nullptr;
-    s->pair_ok = s->g.planes == 3 && L.recon[2] == L.recon[1] + (size_t)s->g.p[1].w * s->g.p[1].h &&
-                 L.recon1[2] == L.recon1[1] + (size_t)s->g.p[1].w * s->g.p[1].h;
     s->mask = (uint8_t *)(base + L.mask);
-    s->tiles = (uint32_t *)(base + L.tiles);
-    s->ctiles = (uint32_t *)(base + L.ctiles);
-    s->tile_gen = (uint32_t *)(base + L.tile_gen);
-    s->ctile_gen = (uint32_t *)(base + L.ctile_gen);
-    for (int p = 0; p < 3; ++p) {
-        const bool has = p < s->g.planes && s->g.levels >= 3;
-        s->ll2[p] = has ? (float *)(base + L.ll2[p]) : nullptr;
-        s->ll2_pitch[p] = has ? s->g.p[p].ll2_pitch : 0;
-    }
-    s->counters = (int *)(base + L.counters);
     s->err = (int *)(base + L.err);
-    for (int p = 0; p < 3; ++p) s->ll2_1[p] = s->ll2[p] ? (float *)(base + L.ll2_1[p]) : nullptr;
-    s->tiles1 = (uint32_t *)(base + L.tiles1);
-    s->ctiles1 = (uint32_t *)(base + L.ctiles1);
-    s->counters1 = (int *)(base + L.counters1);
+    s->n_sets = L.n_sets;
+    s->pair_ok = s->g.planes == 3;
+    for (int k = 0; k < L.n_sets; ++k) {
+        const Layout::Set &A = L.set[k];
+        ViewSet &S = s->set[k];
+        for (int p = 0; p < 3; ++p) {
+            S.recon[p] = p < s->g.planes ? (uint8_t *)(base + A.recon[p]) : nullptr;
+            S.ll2[p] = p < s->g.planes && s->g.levels >= 3 ? (float *)(base + A.ll2[p]) : nullptr;
+        }
+        S.tiles = (uint32_t *)(base + A.tiles);
+        S.ctiles = (uint32_t *)(base + A.ctiles);
+        S.tile_gen = (uint32_t *)(base + A.tile_gen);
+        S.ctile_gen = (uint32_t *)(base + A.ctile_gen);
+        S.counters = (int *)(base + A.counters);
+        s->pair_ok = s->pair_ok && A.recon[2] == A.recon[1] + (size_t)s->g.p[1].w * s->g.p[1].h;
+    }
+    for (int p = 0; p < 3; ++p)
+        s->ll2_pitch[p] = p < s->g.planes && s->g.levels >= 3 ? s->g.p[p].ll2_pitch : 0;
     const size_t tcount = (size_t)s->g.num_frames * s->g.nbpf;
     s->table_host.resize(tcount);
     if (is_paper) {
@@ -880,9 +865,9 @@ int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t devi
     if (e == cudaSuccess && !is_paper && h.n_payload && s->g.wavelet == WV_WAVELET_97 && s->g.quant == 0) {
         const size_t count = (size_t)h.n_payload * s->g.block * s->g.block;
         int max_abs = 0;
-        e = cudaMemsetAsync(s->counters + 8, 0, 4, s->cs);
-        if (e == cudaSuccess) e = payload_max_abs(s->payload, count, s->counters + 8, s->cs);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&max_abs, s->counters + 8, 4, cudaMemcpyDeviceToHost, s->cs);
+        e = cudaMemsetAsync(s->set[0].counters + 8, 0, 4, s->cs);
+        if (e == cudaSuccess) e = payload_max_abs(s->payload, count, s->set[0].counters + 8, s->cs);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&max_abs, s->set[0].counters + 8, 4, cudaMemcpyDeviceToHost, s->cs);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->cs);
         if (e == cudaSuccess && max_abs <= kDzTMax) {
             e = payload_to_deadzone_t(s->payload, count, s->cs);
@@ -890,10 +875,7 @@ int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t devi
             s->gsq.dz_t = 1;
         }
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + L.recon[0], 0, L.tiles - L.recon[0], s->cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + L.recon1[0], 0, L.total - L.recon1[0], s->cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + L.tile_gen, 0, L.err + 64 - L.tile_gen, s->cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + L.ll2_1[0], 0, L.total - L.ll2_1[0], s->cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + L.mask, 0, L.total - L.mask, s->cs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->cs);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -915,18 +897,14 @@ int wv_set_cuda_stream(wv_stream *s, void *cuda_stream) {
 void wv_close_stream(wv_stream *s) {
     if (!s) return;
     cudaStreamSynchronize(s->cs);
-    if (s->aux) {
-        cudaStreamSynchronize(s->aux);
-        cudaStreamDestroy(s->aux);
+    for (ViewSet &S : s->set) {
+        if (S.st) {
+            cudaStreamSynchronize(S.st);
+            cudaStreamDestroy(S.st);
+        }
+        for (cudaEvent_t e : {S.fine, S.free})
+            if (e) cudaEventDestroy(e);
     }
-    if (s->fs) {
-        cudaStreamSynchronize(s->fs);
-        cudaStreamDestroy(s->fs);
-    }
-    for (cudaEvent_t e : {s->ev_fine[0], s->ev_fine[1]})
-        if (e) cudaEventDestroy(e);
-    for (cudaEvent_t e : {s->ev_ready[0], s->ev_ready[1], s->ev_free[0], s->ev_free[1]})
-        if (e) cudaEventDestroy(e);
     if (s->host_payload) cudaFreeHost(s->host_payload);
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     if (s->owns && s->dmem) cudaFree(s->dmem);
@@ -956,7 +934,8 @@ int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float)
     } guard{s, s->decode_mode};
     if (as_float && strip_mode(s) && !strip_float_supported(s->g)) s->decode_mode = 2;
     const Geom &g = active_geom(s);
-    uint8_t *outs[3] = {s->recon[0], s->recon[1], s->recon[2]};
+    const ViewSet &S = s->set[0];
+    uint8_t *outs[3] = {S.recon[0], S.recon[1], S.recon[2]};
     float *f32 = nullptr;
     if (dptr) {
         if (as_float) f32 = (float *)dptr;
@@ -965,8 +944,8 @@ int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float)
     // strips: every tile of the plane, without lists (their count only serves
     // the profile)
     const int all_plane = strip_mode(s) ? plane : -1;
-    if (all_plane < 0 || s->prof) launch_all_tiles(g, plane, s->tiles, s->counters, s->cs);
-    if (all_plane < 0 && split_mode(s)) launch_all_ctiles(g, plane, s->ctiles, s->counters, s->cs);
+    if (all_plane < 0 || s->prof) launch_all_tiles(g, plane, S.tiles, S.counters, s->cs);
+    if (all_plane < 0 && split_mode(s)) launch_all_ctiles(g, plane, S.ctiles, S.counters, s->cs);
     cudaError_t e = run_decode(s, stream_bands(s, frame), outs, f32, as_float ? plane : -1, all_plane);
     mark_sets_used(s);
     if (!dptr) {   // set 0's reconstruction now holds the decode (for wv_resample_at)
@@ -995,13 +974,14 @@ int wv_debug_footprint(wv_stream *s, float yaw, float pitch, float fov, int out_
     const View v = make_view(yaw, pitch, fov, out_w, out_h, g.p[0].w, rows, row0);
     uint8_t *m = s->mask;
     const uint32_t gen = next_gen(s);
-    launch_footprint(g, v, m, s->tile_gen, s->ctile_gen, gen, s->counters, s->cs);
-    launch_select_tiles(g, s->tile_gen, s->ctile_gen, gen, s->tiles, s->ctiles, s->counters, s->cs);
+    const ViewSet &S = s->set[0];
+    launch_footprint(g, v, m, S.tile_gen, S.ctile_gen, gen, S.counters, s->cs);
+    launch_select_tiles(g, S.tile_gen, S.ctile_gen, gen, S.tiles, S.ctiles, S.counters, s->cs);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && mask_host)
         e = cudaMemcpyAsync(mask_host, m, (size_t)g.cells_x * g.cells_y, cudaMemcpyDeviceToHost, s->cs);
     int cnt = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, s->counters, 4, cudaMemcpyDeviceToHost, s->cs);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, S.counters, 4, cudaMemcpyDeviceToHost, s->cs);
     mark_sets_used(s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->cs);
     if (tiles) *tiles = cnt;
@@ -1091,7 +1071,7 @@ int wv_profile_end(wv_stream *s, wv_profile *out) {
         out->launches[k] += 1;
     }
     int cnt = 0;
-    cudaMemcpy(&cnt, s->counters, 4, cudaMemcpyDeviceToHost);
+    cudaMemcpy(&cnt, s->set[0].counters, 4, cudaMemcpyDeviceToHost);
     out->tiles = cnt;
     s->prof = false;
     s->ev_used = 0;

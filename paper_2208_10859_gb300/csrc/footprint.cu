@@ -137,6 +137,8 @@ __device__ __forceinline__ bool cell_needed_eye(const View &v, const Frustum &f,
     return cell_needed(f, eq_w, v.rows, nc, cx, cy - c0);
 }
 
+// mask: or null (only wv_debug_footprint reads it; viewports in flight at the
+// same time would write it over one another).
 __global__ void k_footprint(View v, Frustum f, Geom g, uint8_t *__restrict__ mask,
                             uint32_t *__restrict__ tile_gen, uint32_t *__restrict__ ctile_gen,
                             uint32_t gen, int *counters) {
@@ -145,7 +147,7 @@ __global__ void k_footprint(View v, Frustum f, Geom g, uint8_t *__restrict__ mas
     if (cx == 0 && cy == 0) counters[0] = counters[1] = counters[2] = 0;   // tile counts of this viewport
     if (cx >= g.cells_x || cy >= g.cells_y) return;
     const bool hit = cell_needed_eye(v, f, g.p[0].w, cx, cy);
-    mask[cy * g.cells_x + cx] = hit ? 1 : 0;
+    if (mask) mask[cy * g.cells_x + cx] = hit ? 1 : 0;
     if (hit) stamp_cell(g, cx, cy, tile_gen, ctile_gen, gen);
 }
 

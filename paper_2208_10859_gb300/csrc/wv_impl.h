@@ -384,6 +384,32 @@ int encode_paper(const Geom &g, const void *const *planes, void *scratch, size_t
 
 }  // namespace wv
 
+namespace wv {
+
+// The buffers of one viewport in flight and its internal stream.  A chain of
+// kernels on `st` (footprint, selection, coarse pass, fine pass) fills the
+// set, cs waits for it (`fine`) and resamples, and the set's next chain waits
+// for that (`free`): the chains of consecutive viewports overlap each other
+// and the resampling.  Frames too small to fill the chip (kFineStrips) are
+// bound by the length of that chain, not by its work, and take four sets,
+// larger ones three.  Four viewports (eight of 8192^2) with two sets, three,
+// four: 2880 x 1440 126, 116, 95 us; 4096^2 stereo 185, 178, 156; 6144 x 3072
+// 165, 159, 143; 8192^2 913, 866, 866.  Six for the small ones gave nothing.
+// (With three internal streams shared by two sets, the coarse passes of
+// consecutive viewports ran one after the other: 143, 213, 174, 957 us.)
+constexpr int kViewSets = 4, kViewSetsLarge = 3;
+struct ViewSet {
+    uint32_t *tiles = nullptr, *ctiles = nullptr;        // tile lists
+    uint32_t *tile_gen = nullptr, *ctile_gen = nullptr;  // stamps
+    int *counters = nullptr;
+    float *ll2[3] = {nullptr, nullptr, nullptr};
+    uint8_t *recon[3] = {nullptr, nullptr, nullptr};
+    cudaStream_t st = nullptr;
+    cudaEvent_t fine = nullptr, free = nullptr;
+};
+
+}  // namespace wv
+
 struct wv_stream {
     // g: geometry of the default decode (strip tiles when strip_eligible,
     // else square tiles); gsq: square 128-sample tiles (decode modes 1, 2)
@@ -397,41 +423,20 @@ struct wv_stream {
     size_t dbytes = 0;
     int16_t *payload = nullptr;
     int32_t *table = nullptr;
-    uint8_t *recon[3] = {nullptr, nullptr, nullptr};
     uint8_t *mask = nullptr;
-    uint32_t *tiles = nullptr;
-    uint32_t *tile_gen = nullptr;
-    uint32_t *ctile_gen = nullptr;
-    uint32_t *ctiles = nullptr;
     uint32_t gen = 0;   // viewport generation (stamps in tile_gen / ctile_gen)
-    float *ll2[3] = {nullptr, nullptr, nullptr};
     int ll2_pitch[3] = {0, 0, 0};
     int decode_mode = 0;   // 0: default (strip fine pass), 1: all levels fused per square tile,
                            // 2: coarse pass + square-tile fine pass
     bool pair_ok = false;  // recon[1], recon[2] adjacent: chroma can be held in alternating groups
-    int *counters = nullptr;
     int *err = nullptr;
-    // A second set of per-viewport buffers (tile lists, counters, LL_2
-    // planes): consecutive viewports alternate between the sets, so the
-    // footprint, selection and coarse pass of a viewport (on the internal
-    // stream `aux`) run while the previous viewport's fine pass and
-    // resampling (on cs) are still executing.  Set 0 is the fields above.
-    // The sets also hold a reconstruction each: a viewport's fine pass (on
-    // the internal stream `fs`) writes one while the previous viewport's
-    // resampling (on cs) reads the other.
-    uint32_t *tiles1 = nullptr, *ctiles1 = nullptr;
-    int *counters1 = nullptr;
-    float *ll2_1[3] = {nullptr, nullptr, nullptr};
-    uint8_t *recon1[3] = {nullptr, nullptr, nullptr};
-    int slot = 0;
+    // Consecutive viewports take the sets in turn; work on cs itself uses set 0.
+    wv::ViewSet set[wv::kViewSets];
+    int n_sets = 1;
+    int slot = 0;            // the set of the next overlapped viewport
     int cur = 0;             // the set whose reconstruction holds the last decode
     bool pending = false;    // the last decode's set is released after its resampling on cs
     bool overlap = true;
-    cudaStream_t aux = nullptr;
-    cudaStream_t fs = nullptr;
-    cudaEvent_t ev_ready[2] = {nullptr, nullptr};   // set k's coarse pass done (aux)
-    cudaEvent_t ev_fine[2] = {nullptr, nullptr};    // set k's fine pass done (fs)
-    cudaEvent_t ev_free[2] = {nullptr, nullptr};    // cs no longer reads set k
     uint64_t n_payload = 0;
     void *host_payload = nullptr;   // WV_OPEN_HOST_PAYLOAD: pinned, mapped coefficient store
     std::vector<int32_t> table_host;
