@@ -11,9 +11,9 @@
 //   tile_gen  uint32 [tiles]            generation that last selected a tile
 //   ctile_gen uint32 [coarse tiles]      generation that last listed a coarse tile
 //   ctiles    uint32 [coarse tiles]      coarse tiles the selected tiles need
-//   counters  int32 [16]                 [0] = tile count, [1] = coarse tile count,
-//                                        [2] = strip tiles taken (strip kernel)
+//   counters  int32 [16]                 [0] = tile count, [1] = coarse tile count
 //   err       int32                      first device-side error code
+// (recon, ll2, lists, stamps and counters once per viewport set)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -172,9 +172,10 @@ struct TileArgs {
 };
 
 // Every tile of one plane instead of a list (n > 0: n tiles, nx per row).  A
-// kernel argument of its own: a kernel that chooses between a field of a
-// struct argument and a value in memory may read the wrong one's address
-// space, or keeps a copy of the struct in local memory.
+// kernel argument of its own: with the count a field of TileArgs, choosing
+// between it and the list's count in memory made the compiler keep a 1.3 KB
+// copy of TileArgs per thread in local memory, and with TileArgs declared
+// __grid_constant__ the count was read from an invalid address.
 struct AllTiles {
     int n, plane, nx;
 #ifdef __CUDACC__
@@ -292,6 +293,7 @@ int viewable_strips(const wv_stream_desc &d);   // 64-row strips of what an eye 
 
 Bands frame_bands(const Geom &g, int frame);
 View make_view(float yaw, float pitch, float fov, int out_w, int out_h, int eq_w, int eq_h, int row0 = 0);
+int decode_full_overlapped(wv_stream *s, const Bands &b, uint8_t *const *outs, float *f32, int plane);
 int eye_view(const Geom &g, int eye, int *row0, int *rows);   // WV_ERR_ARG for an invalid eye
 Frustum make_frustum(const View &v);
 
