@@ -86,6 +86,7 @@ struct Wave {
     size_t lists_c[kClasses], lists_f[kClasses], lists_s[kClasses];
     int smem[kClasses];    // dynamic shared memory of each class's decode (0: class absent)
     bool strip[kClasses];  // the class has strip surfaces in this wave
+    int q0[kClasses], qn[kClasses];   // rows of the request table by class
     int max_cx, max_cy, max_stamps, max_w, max_h;
 };
 
@@ -235,13 +236,20 @@ int plan_batch(const wv_batch *b, const wv_request *reqs, int n, Plan &P) {
         }
         if (m > 0) P.waves.push_back(Wave{s0, m});
     }
-    // request table: by wave, caller order inside a wave
+    // request table: by wave and class, caller order inside a class
     P.order.clear();
     for (Wave &W : P.waves) {
         W.r0 = (int)P.order.size();
         for (int i = 0; i < n; ++i)
             if (P.req_surface[i] >= W.s0 && P.req_surface[i] < W.s1) P.order.push_back(i);
         W.r1 = (int)P.order.size();
+        auto cls = [&](int i) { return P.surf[P.req_surface[i]].cls; };
+        std::stable_sort(P.order.begin() + W.r0, P.order.end(), [&](int i, int j) { return cls(i) < cls(j); });
+        for (int c = 0; c < kClasses; ++c) W.q0[c] = W.qn[c] = 0;
+        for (int k = W.r1 - 1; k >= W.r0; --k) {
+            W.q0[cls(P.order[k])] = k;
+            W.qn[cls(P.order[k])] += 1;
+        }
     }
     // arena: error word | job tables | counters of every wave | wave region
     // (stamps | lists | per-surface planes, reused by every wave).  The error
@@ -474,9 +482,10 @@ cudaError_t enqueue(wv_batch *b, const Plan &P, int n, cudaStream_t cs, bool tim
         }
         launch_select_batch(surfs + W.s0, m, W.max_stamps, lists, ctr, cs);
         if (timed) cudaEventRecord(ev[2], cs);
-        // The classes are independent until the resampling: each is a branch of
-        // the captured graph (coarse tiles, then its strip tiles), so the tail
-        // of one class's launch overlaps the others' work.
+        // The classes are independent: each is a branch of the captured graph
+        // (coarse tiles, strip tiles, resampling), so the tail of one class's
+        // launch overlaps the others' work, and the resampling of one (bound
+        // by its gathers) the strips of another (bound by their chains).
         std::vector<int> classes;
         for (int c = 0; c < kClasses; ++c)
             if (W.smem[c]) classes.push_back(c);
@@ -486,12 +495,14 @@ cudaError_t enqueue(wv_batch *b, const Plan &P, int n, cudaStream_t cs, bool tim
             const cudaStream_t bs = branch && k > 0 ? b->side[k - 1] : cs;
             if (bs != cs) e = cudaStreamWaitEvent(bs, b->fork, 0);
             if (e == cudaSuccess) e = launch_class(b, P, W, classes[k], lists, bs);
+            if (e == cudaSuccess && branch && W.qn[classes[k]] > 0)
+                launch_resample_batch(rq + W.q0[classes[k]], W.qn[classes[k]], W.max_w, W.max_h, bs);
             if (bs != cs && e == cudaSuccess) e = cudaEventRecord(b->join, bs);
             if (bs != cs && e == cudaSuccess) e = cudaStreamWaitEvent(cs, b->join, 0);
         }
         if (e != cudaSuccess) return e;
         if (timed) cudaEventRecord(ev[3], cs);
-        launch_resample_batch(rq + W.r0, nr, W.max_w, W.max_h, cs);
+        if (!branch) launch_resample_batch(rq + W.r0, nr, W.max_w, W.max_h, cs);
         if (timed) cudaEventRecord(ev[4], cs);
     }
     return cudaGetLastError();
@@ -512,6 +523,8 @@ std::vector<long long> shape_key(const wv_batch *b, const Plan &P, int n) {
             k.push_back((long long)W.lists_f[c]);
             k.push_back((long long)W.lists_s[c]);
             k.push_back(W.strip[c] ? 1 : 0);
+            k.push_back(W.q0[c]);
+            k.push_back(W.qn[c]);
         }
     }
     return k;
