@@ -539,9 +539,11 @@ __global__ void __launch_bounds__(net_threads(BWD), 1) k_net(NetArgs a) {
 // Bound: the MMAs' reads of A (4 KB per 16 pixels and dx) and the 128 bytes
 // per pixel from HBM, about 20 us each for 16 x 256^2 pixels; two CTAs per SM
 // so that one's loads run under the other's MMAs (one CTA with two operand
-// buffers: 88 us, too few warps issuing loads).  Measured
-// 71 us; the form with both operands transposed through shared memory by the
-// threads took 434 us.
+// buffers: 88 us, too few warps issuing loads).  One
+// layer alone takes 70 us (with both operands transposed through shared memory
+// by the threads 434), the three of a step in one launch 190: a third of the
+// CTAs' fills, drains and gradient additions, which go out four floats at a
+// time.
 constexpr int kWRowsT = 4;                              // dz rows per tile
 constexpr int kWThreads = 256;
 constexpr int kWAct = (kWRowsT + 3) * kSlot;            // kWRowsT + 2 rows, one more that the last M reads
@@ -555,9 +557,22 @@ __device__ __forceinline__ void cp_async16(uint8_t *dst, const void *src, bool f
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restrict__ act, const bf16 *__restrict__ dz,
-                                                           int n, int h, int w, float *dW, float *db, int *err) {
+// The three layers of a step, one of them per CTA: layer blockIdx.x % layers.
+constexpr int kMidLayers = 3;
+struct WgradArgs {
+    const bf16 *act[kMidLayers], *dz[kMidLayers];
+    float *dW[kMidLayers], *db[kMidLayers];   // dW 16-byte aligned
+    int layers, n, h, w;
+    int *err;
+};
+
+__global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(WgradArgs args) {
     extern __shared__ __align__(128) uint8_t sm[];
+    const int layer = blockIdx.x % args.layers, cta = blockIdx.x / args.layers, ctas = gridDim.x / args.layers;
+    const bf16 *__restrict__ act = args.act[layer], *__restrict__ dz = args.dz[layer];
+    float *dW = args.dW[layer], *db = args.db[layer];
+    int *err = args.err;
+    const int n = args.n, h = args.h, w = args.w;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ float sBias[kC];
@@ -605,7 +620,7 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restri
             if (tid == 0) record_error(err, WV_ERR_TIMEOUT);
         }
     };
-    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+    for (int it = cta; it < total; it += ctas) {
         if (!first) wait_mma();
         if (!ok) break;
         load(it);
@@ -668,7 +683,8 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(const bf16 *__restri
             if ((tid & 31) < 4) atomicAdd(&sBias[8 * (tid & 3) + e], v);
         }
         __syncthreads();
-        for (int i = tid; i < kC * kC * 9; i += kWThreads) atomicAdd(dW + i, out[i]);
+        for (int i = tid; i < kC * kC * 9 / 4; i += kWThreads)
+            atomicAdd(reinterpret_cast<float4 *>(dW) + i, reinterpret_cast<const float4 *>(out)[i]);
         if (tid < kC) atomicAdd(db + tid, sBias[tid]);
     }
     umma::fence_before_sync();
@@ -922,13 +938,12 @@ cudaError_t launch_net(NetArgs &a, cudaStream_t cs) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_wgrad_mid(const bf16 *act, const bf16 *dz, int n, int h, int w, float *dW, float *db, int *err,
-                             cudaStream_t cs) {
+cudaError_t launch_wgrad_mid(const WgradArgs &a, cudaStream_t cs) {
     cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_wgrad_mid), kWSmem);
     if (e != cudaSuccess) return e;
-    const int total = n * ((h + kWRowsT - 1) / kWRowsT) * ((w + kTilePx - 1) / kTilePx);
-    const int grid = std::max(1, std::min(total, 2 * sm_count()));
-    k_wgrad_mid<<<grid, kWThreads, kWSmem, cs>>>(act, dz, n, h, w, dW, db, err);
+    const int total = a.n * ((a.h + kWRowsT - 1) / kWRowsT) * ((a.w + kTilePx - 1) / kTilePx);
+    const int ctas = std::max(1, std::min(total, 2 * sm_count() / a.layers));   // of one layer
+    k_wgrad_mid<<<ctas * a.layers, kWThreads, kWSmem, cs>>>(a);
     return cudaGetLastError();
 }
 
@@ -989,10 +1004,23 @@ cudaError_t forward_backward(wv_cnn *c, const float *x, const float *t, int n, i
         a.out[s] = c->g[3 - s];
     }
     e = launch_net<true>(a, cs);
+    if (e != cudaSuccess) return e;
     float *G = c->grads;
-    if (e == cudaSuccess) e = launch_wgrad_edge(c->dz5, c->act[3], 0, n, h, w, G + off_w(4), G + off_b(4), cs);
-    for (int l = 3; l >= 1 && e == cudaSuccess; --l)
-        e = launch_wgrad_mid(c->act[l - 1], c->g[l], n, h, w, G + off_w(l), G + off_b(l), c->err, cs);
+    WgradArgs m;
+    memset(&m, 0, sizeof(m));
+    m.layers = kMidLayers;
+    m.n = n;
+    m.h = h;
+    m.w = w;
+    m.err = c->err;
+    for (int l = 1; l <= kMidLayers; ++l) {
+        m.act[l - 1] = c->act[l - 1];
+        m.dz[l - 1] = c->g[l];
+        m.dW[l - 1] = G + off_w(l);
+        m.db[l - 1] = G + off_b(l);
+    }
+    e = launch_wgrad_edge(c->dz5, c->act[3], 0, n, h, w, G + off_w(4), G + off_b(4), cs);
+    if (e == cudaSuccess) e = launch_wgrad_mid(m, cs);
     if (e == cudaSuccess) e = launch_wgrad_edge(x, c->g[0], 1, n, h, w, G + off_w(0), G + off_b(0), cs);
     return e;
 }
