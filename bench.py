@@ -693,7 +693,7 @@ def cpu_baseline_leg(frames, poses, size, n_poses):
     parity = {"plane": f"luma of frame 0, {size}x{size}, encoded by the oracle", "samples": size * size,
               "max_abs_err_levels": err, "regression_bound_levels": 5e-4, "tolerance_levels": 1e-4 * 255,
               "u8_samples_differing": mism,
-              "note": "float32 whole-plane decode (square-tile passes) against the fp64 oracle in 8-bit levels; "
+              "note": "float32 whole-plane decode against the fp64 oracle in 8-bit levels; "
                       "8-bit samples (strip fine pass) differ only where the fp64 value lies within the float "
                       "error of a rounding boundary"}
     return {"value": res[cores][0], "unit": UNIT, "cores": cores, "kind": "oracle", "cpu_model": model,

@@ -104,7 +104,7 @@ int wv_stream_query(const void *bytes, size_t n, wv_stream_desc *desc,
 
 /* Open a stream: validate the bytes, copy the block table and the coefficient
  * payload to the device and set up per-stream decode scratch (reconstruction
- * planes, mask, two sets of tile lists and LL_2 planes).  CDF 9/7 dead-zone
+ * planes, LL_2 planes and tile lists of up to four viewports in flight, mask).  CDF 9/7 dead-zone
  * codes are rewritten on the device as 2q + sign(q) when every |q| <= 8191
  * (one pass over the payload; decoded results are unchanged).  The call
  * synchronises cuda_stream before it returns.  device_mem is a device
@@ -297,7 +297,7 @@ int wv_batch_set_sharing(wv_batch *b, int on);
 
 /* on = 1 (default): decode targets whose streams the strip fine pass takes
  * (dead-zone codes, three or more levels, one or two coefficient frames)
- * decode levels 2 and 1 as 224 x 64 strips (k_strip_batch, foveation
+ * decode levels 2 and 1 as 224-column strips (k_strip_batch, foveation
  * included), after the class's coarse tiles; on = 0: square tiles for
  * every target.  Outputs are identical either way. */
 int wv_batch_set_strips(wv_batch *b, int on);
@@ -497,7 +497,7 @@ int wv_decode_viewport_filtered(wv_stream *s, int frame, float yaw, float pitch,
  * for the lossless workload and for parity checks.  dptr receives width x
  * height samples of the plane, row-major and tightly packed: uint8
  * (as_float = 0) or float32 values before rounding (as_float = 1, 8-bit
- * units, DC offset included; always the square-tile passes).  dptr == NULL
+ * units, DC offset included).  dptr == NULL
  * decodes into the stream's own reconstruction plane (as uint8, in the
  * layout of the current decode mode) for wv_resample_at. */
 int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float);
@@ -594,8 +594,8 @@ int wv_request_bytes(const wv_request *r, unsigned long long *cone, unsigned lon
 typedef struct {
     double ms[8];        /* footprint, select tiles, coarse decode, fine decode, resample */
     int launches[8];
-    int tiles;           /* tiles decoded by the last viewport (an edge strip
-                            counts as its two halves) */
+    int tiles;           /* tiles decoded by the last viewport (a strip listed
+                            as two halves counts as two) */
 } wv_profile;
 
 /* Start recording: the following decode calls on s record events around
@@ -611,9 +611,10 @@ int wv_launches_per_viewport(const wv_stream *s);
 /* Tile-decode organisation.  Mode 0 (default): levels L..3 of the needed
  * coarse tiles go into float LL_2 planes in one kernel (streams of three or
  * more levels), then levels 2 and 1 of the needed output tiles in a second;
- * for dead-zone streams of three or more levels the second kernel streams
- * each 224-column strip of the region down its rows in one warp (strip
- * tiles; 8-bit output only: float whole-plane decodes take mode 2), with
+ * for streams of three or more levels the second kernel streams each
+ * 224-column strip of the region down its rows in one warp (strip tiles;
+ * float whole-plane decodes of record streams and of 9/7 codes above 8191
+ * take mode 2), with
  * the reconstruction's chroma held as alternating Cb and Cr groups of four
  * samples; otherwise it decodes square 128-sample tiles.  Mode 1: all
  * levels of each square output tile in one kernel, repeating the coarse
