@@ -699,15 +699,23 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(WgradArgs args) {
 // tap flipped (T[p + tap - 1] P[p] = T[q] P[q - (tap - 1)]).  Four lanes hold a
 // pixel's channels (one 16-byte load each) and walk along a run of a row, eight
 // runs side by side in a warp, with the 3 x 3 window of P sliding in registers:
-// 4 loads and 36 packed FMAs for 8 pixels.  46 us for 16 x 256^2 pixels; staged
-// in shared memory, with two loads per FMA, it took 138 and 153 us.
+// 4 loads and 36 packed FMAs for 8 pixels.
+// Bound: latency.  With the tensor's loads in the loop (no registers left to
+// fetch ahead) it took 47 us for 16 x 256^2 pixels, 2 us for every three pixels
+// of a lane; each lane now copies its own pixels to shared memory kEStages - 1
+// steps of three ahead: 39 us.  (Staged in shared memory per CTA, with two loads
+// per FMA, 138 and 153 us.)
 constexpr int kEWarps = 8;
 constexpr int kERunMax = 33;     // pixels per run, a multiple of the window's 3 columns
+constexpr int kEStages = 6;
+constexpr int kEStage = 3 * 32 * 16;                      // bytes of a warp's step
+constexpr int kESmem = kEWarps * kEStages * kEStage;
 
 __global__ void __launch_bounds__(32 * kEWarps, 2) k_wgrad_edge(const float *__restrict__ plane,
                                                                const bf16 *__restrict__ act, int first_layer, int n, int h,
                                                                int w, int run, int runs, float *dW, float *db) {
     __shared__ float sum[kEWarps][kC * 10];   // [c][tap], then the bias
+    extern __shared__ __align__(128) uint8_t sm[];
     const int tid = threadIdx.x, lane = tid & 31, q = lane & 3, warp = tid >> 5;
     float2 acc[9][4] = {}, bias[4] = {};
     float centre = 0.f;
@@ -724,16 +732,30 @@ __global__ void __launch_bounds__(32 * kEWarps, 2) k_wgrad_edge(const float *__r
             v[1] = in ? __ldg(row + x) : 0.f;
             v[2] = in && dn ? __ldg(row + w + x) : 0.f;
         };
+        // the lane's pixels xa + 3 g .. + 2 into its slots of stage g mod kEStages
+        uint8_t *ring = sm + (size_t)warp * kEStages * kEStage + lane * 16;
+        auto fetch = [&](int g) {
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const int x = xa + 3 * g + r;
+                const bool in = 3 * g < run && x < xe;
+                cp_async16(ring + (g % kEStages) * kEStage + r * 512, reinterpret_cast<const uint8_t *>(in ? t + 4 * (size_t)x : t), in);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        for (int g = 0; g < kEStages - 1; ++g) fetch(g);
         float p[3][3];   // window columns x - 1, x, x + 1 (rotating)
         load(xa - 1, p[0]);
         load(xa, p[1]);
 #pragma unroll 1
-        for (int k0 = 0; k0 < run; k0 += 3)
+        for (int k0 = 0, g = 0; k0 < run; k0 += 3, ++g) {
+            fetch(g + kEStages - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kEStages - 1) : "memory");
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
                 const int x = xa + k0 + r;
                 load(x + 1, p[(r + 2) % 3]);
-                const uint4 u = x < xe ? __ldg(t + 4 * (size_t)x) : make_uint4(0u, 0u, 0u, 0u);
+                const uint4 u = *reinterpret_cast<const uint4 *>(ring + (g % kEStages) * kEStage + r * 512);
                 const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
                 float2 tv[4];
 #pragma unroll
@@ -750,6 +772,9 @@ __global__ void __launch_bounds__(32 * kEWarps, 2) k_wgrad_edge(const float *__r
                     for (int e = 0; e < 4; ++e) acc[k][e] = __ffma2_rn(tv[e], p2, acc[k][e]);
                 }
             }
+        }
+        // the fills past the run's end, before the next run's copies into the same slots
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     // over the warp's eight runs, then over the CTA's warps
     auto reduce = [&](float v) {
@@ -954,7 +979,9 @@ cudaError_t launch_wgrad_edge(const float *plane, const bf16 *act, int first, in
     const int run = 3 * ((w + 24 * runs - 1) / (24 * runs));
     const int total = n * h * runs;
     const int grid = std::max(1, std::min((total + kEWarps - 1) / kEWarps, 2 * sm_count()));
-    k_wgrad_edge<<<grid, 32 * kEWarps, 0, cs>>>(plane, act, first, n, h, w, run, runs, dW, db);
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_wgrad_edge), kESmem);
+    if (e != cudaSuccess) return e;
+    k_wgrad_edge<<<grid, 32 * kEWarps, kESmem, cs>>>(plane, act, first, n, h, w, run, runs, dW, db);
     return cudaGetLastError();
 }
 
