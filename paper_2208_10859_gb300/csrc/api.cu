@@ -286,6 +286,7 @@ cudaError_t take_lane(int device, Lane *l) {
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
         std::vector<Lane> &v = idle_lanes()[device];
+        v.reserve(kLanesKept);   // give_lane never allocates
         if (!v.empty()) {
             *l = v.back();
             v.pop_back();
@@ -318,8 +319,11 @@ void give_lane(int device, const Lane &l) {
 cudaError_t ensure_set(wv_stream *s, int k) {
     ViewSet &S = s->set[k];
     if (S.st) return cudaSuccess;
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev != s->device) return cudaErrorInvalidDevice;   // a new lane would be the other device's
     Lane l;
-    cudaError_t e = take_lane(s->device, &l);
+    if (e == cudaSuccess) e = take_lane(s->device, &l);
     if (e == cudaSuccess && (e = cudaEventRecord(l.free, s->cs)) != cudaSuccess) give_lane(s->device, l);
     if (e != cudaSuccess) {
         cudaGetLastError();
