@@ -467,7 +467,9 @@ int wv_cnn_set_params(wv_cnn *c, const float *params_host);
 int wv_cnn_get_state(wv_cnn *c, float *m_host, float *v_host, int *steps);
 int wv_cnn_set_state(wv_cnn *c, const float *m_host, const float *v_host, int steps);
 
-/* y = network(x) for n images of h x w (device float planes). */
+/* y = network(x) for n images of h x w (device float planes).  y_dev may be
+ * x_dev or overlap it: the input is then copied aside first (stream-ordered
+ * device memory for one copy of x; WV_ERR_OOM when there is none). */
 int wv_cnn_forward(wv_cnn *c, const float *x_dev, float *y_dev, int n, int h, int w, void *cuda_stream);
 
 /* Loss mean((y - t)^2) and its gradient with respect to every parameter

@@ -1148,11 +1148,31 @@ int wv_cnn_set_state(wv_cnn *c, const float *m_host, const float *v_host, int st
 
 int wv_cnn_forward(wv_cnn *c, const float *x_dev, float *y_dev, int n, int h, int w, void *cuda_stream) {
     if (!c || !x_dev || !y_dev || check_dims(n, h, w) != WV_OK) return WV_ERR_ARG;
+    cudaStream_t cs = (cudaStream_t)cuda_stream;
+    // Filtering in place: a CTA stores y while others still read x around
+    // their own tiles, so where the planes overlap the network reads a copy of
+    // x.  The copy is the call's own (stream-ordered memory), so that calls on
+    // several streams do not share it and a captured call holds it itself.
+    const size_t bytes = sizeof(float) * (size_t)n * h * w;
+    const uintptr_t xa = (uintptr_t)x_dev, ya = (uintptr_t)y_dev;
+    float *copy = nullptr;
+    if (xa < ya + bytes && ya < xa + bytes) {
+        if (cudaMallocAsync((void **)&copy, bytes, cs) != cudaSuccess) {
+            cudaGetLastError();
+            return WV_ERR_OOM;
+        }
+    }
     NetArgs fin;
     memset(&fin, 0, sizeof(fin));
     fin.mode = kOut;
     fin.y = y_dev;
-    return forward(c, x_dev, n, h, w, fin, (cudaStream_t)cuda_stream) == cudaSuccess ? WV_OK : WV_ERR_CUDA;
+    cudaError_t e = copy ? cudaMemcpyAsync(copy, x_dev, bytes, cudaMemcpyDeviceToDevice, cs) : cudaSuccess;
+    if (e == cudaSuccess) e = forward(c, copy ? copy : x_dev, n, h, w, fin, cs);
+    if (copy) {
+        const cudaError_t ef = cudaFreeAsync(copy, cs);
+        if (e == cudaSuccess) e = ef;
+    }
+    return e == cudaSuccess ? WV_OK : WV_ERR_CUDA;
 }
 
 int wv_cnn_gradients(wv_cnn *c, const float *x_dev, const float *t_dev, int n, int h, int w, float *grads_host,
