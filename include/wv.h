@@ -499,9 +499,11 @@ int wv_decode_viewport_filtered(wv_stream *s, int frame, float yaw, float pitch,
  * for the lossless workload and for parity checks.  dptr receives width x
  * height samples of the plane, row-major and tightly packed: uint8
  * (as_float = 0) or float32 values before rounding (as_float = 1, 8-bit
- * units, DC offset included).  dptr == NULL
- * decodes into the stream's own reconstruction plane (as uint8, in the
- * layout of the current decode mode) for wv_resample_at. */
+ * units, DC offset included).  Floats start at a multiple of 4 bytes, uint8
+ * planes at a multiple of 2 (WV_ERR_ARG otherwise; those not at a multiple of
+ * 4 take the square-tile passes).  dptr == NULL decodes into the stream's own
+ * reconstruction plane (as uint8, in the layout of the current decode mode)
+ * for wv_resample_at. */
 int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float);
 
 /* Decode one whole plane without allocating any device memory.  The paper

@@ -1007,14 +1007,16 @@ int wv_decode_full(wv_stream *s, int frame, int plane, void *dptr, int as_float)
     if (!s || frame < 0 || frame >= s->g.num_frames || plane < 0 || plane >= s->g.planes)
         return WV_ERR_ARG;
     if (!dptr && as_float) return WV_ERR_ARG;
-    // float output of streams the float strip kernels do not take runs the
-    // square-tile passes (the same arithmetic per sample)
+    if ((uintptr_t)dptr % (as_float ? 4 : 2)) return WV_ERR_ARG;   // the square tiles store byte pairs
+    // Byte planes off a word boundary (strips store words) and float output of
+    // streams the float strip kernels do not take run the square-tile passes
+    // (the same arithmetic per sample).
     struct ModeGuard {
         wv_stream *s;
         int saved;
         ~ModeGuard() { s->decode_mode = saved; }
     } guard{s, s->decode_mode};
-    if (as_float && strip_mode(s) && !strip_float_supported(s->g)) s->decode_mode = 2;
+    if (strip_mode(s) && (as_float ? !strip_float_supported(s->g) : (uintptr_t)dptr % 4 != 0)) s->decode_mode = 2;
     const Geom &g = active_geom(s);
     const ViewSet &S = s->set[0];
     uint8_t *outs[3] = {S.recon[0], S.recon[1], S.recon[2]};
