@@ -357,7 +357,11 @@ typedef struct {
     int slots;             /* batches in flight at once (one CUDA stream and
                               batch context each), 1..16 */
     int max_batch;         /* requests per batch, >= 1 */
-    size_t cache_bytes;    /* device bytes for resident streams; 0 = no limit */
+    size_t cache_bytes;    /* device bytes for resident streams; 0 = no limit.
+                              A resident stream takes at most what
+                              wv_stream_query says: the server decodes in
+                              batches and leaves out the scratch of a third
+                              and fourth viewport in flight */
     size_t arena_bytes;    /* device bytes for the batch contexts of all
                               slots; 0 = the free device memory minus
                               reserve_bytes */

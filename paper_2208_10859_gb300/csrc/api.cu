@@ -124,9 +124,9 @@ struct Layout {
     } set[kViewSets];   // the buffers of the viewports in flight
 };
 
-// Device layout of a stream; tile lists and stamps hold the larger tile count
-// of the two geometries.
-Layout layout(const Geom &g0, const Geom &gsq, uint64_t n_payload) {
+// Device layout of a stream with at most max_sets buffer sets; tile lists and
+// stamps hold the larger tile count of the two geometries.
+Layout layout(const Geom &g0, const Geom &gsq, uint64_t n_payload, int max_sets) {
     Geom g = g0;
     g.total_tiles = std::max(g0.total_tiles, gsq.total_tiles);
     // tile lists: an edge strip is listed as two half strips
@@ -142,7 +142,7 @@ Layout layout(const Geom &g0, const Geom &gsq, uint64_t n_payload) {
     L.err = o;
     o = align256(o + 64);
     // one viewport at a time without a coarse pass (decode_region)
-    L.n_sets = g.levels < 3 ? 1 : g.strip && g.th == 32 ? kViewSets : kViewSetsLarge;
+    L.n_sets = std::min(max_sets, g.levels < 3 ? 1 : g.strip && g.th == 32 ? kViewSets : kViewSetsLarge);
     for (int k = 0; k < L.n_sets; ++k) {
         Layout::Set &S = L.set[k];
         for (int p = 0; p < 3; ++p) {
@@ -815,6 +815,24 @@ int wv_stream_query(const void *bytes, size_t n, wv_stream_desc *desc, size_t *d
 }
 
 int wv_stream_query_ex(const void *bytes, size_t n, int flags, wv_stream_desc *desc, size_t *device_bytes) {
+    return query_stream(bytes, n, flags, kViewSets, desc, device_bytes);
+}
+
+int wv_open_stream(const void *bytes, size_t n, void *device_mem, size_t device_bytes,
+                   void *cuda_stream, wv_stream **out) {
+    return wv_open_stream_ex(bytes, n, device_mem, device_bytes, cuda_stream, 0, out);
+}
+
+int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t device_bytes,
+                      void *cuda_stream, int flags, wv_stream **out) {
+    return open_stream(bytes, n, device_mem, device_bytes, cuda_stream, flags, kViewSets, out);
+}
+
+}  // extern "C"
+
+namespace wv {
+
+int query_stream(const void *bytes, size_t n, int flags, int max_sets, wv_stream_desc *desc, size_t *device_bytes) {
     if (flags & ~WV_OPEN_HOST_PAYLOAD) return WV_ERR_ARG;
     const bool host_payload = (flags & WV_OPEN_HOST_PAYLOAD) != 0;
     wv_stream_desc d;
@@ -827,7 +845,7 @@ int wv_stream_query_ex(const void *bytes, size_t n, int flags, wv_stream_desc *d
         if (device_bytes) {
             Geom g, gsq;
             stream_geoms(d, info.n_slots, &g, &gsq);
-            *device_bytes = layout(g, gsq, host_payload ? 0 : info.n_slots).total;
+            *device_bytes = layout(g, gsq, host_payload ? 0 : info.n_slots, max_sets).total;
         }
         return WV_OK;
     }
@@ -837,18 +855,13 @@ int wv_stream_query_ex(const void *bytes, size_t n, int flags, wv_stream_desc *d
     if (device_bytes) {
         Geom g, gsq;
         stream_geoms(d, h.n_payload, &g, &gsq);
-        *device_bytes = layout(g, gsq, host_payload ? 0 : h.n_payload).total;
+        *device_bytes = layout(g, gsq, host_payload ? 0 : h.n_payload, max_sets).total;
     }
     return WV_OK;
 }
 
-int wv_open_stream(const void *bytes, size_t n, void *device_mem, size_t device_bytes,
-                   void *cuda_stream, wv_stream **out) {
-    return wv_open_stream_ex(bytes, n, device_mem, device_bytes, cuda_stream, 0, out);
-}
-
-int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t device_bytes,
-                      void *cuda_stream, int flags, wv_stream **out) {
+int open_stream(const void *bytes, size_t n, void *device_mem, size_t device_bytes, void *cuda_stream, int flags,
+                int max_sets, wv_stream **out) {
     if (!out) return WV_ERR_ARG;
     *out = nullptr;
     if (flags & ~WV_OPEN_HOST_PAYLOAD) return WV_ERR_ARG;
@@ -872,7 +885,7 @@ int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t devi
     cudaGetDevice(&s->device);
     s->cs = (cudaStream_t)cuda_stream;
     s->n_payload = h.n_payload;
-    const Layout L = layout(s->g, s->gsq, host_payload ? 0 : h.n_payload);
+    const Layout L = layout(s->g, s->gsq, host_payload ? 0 : h.n_payload, max_sets);
     const size_t payload_bytes = (size_t)h.n_payload * s->g.block * s->g.block * 2;
     if (host_payload && payload_bytes) {
         // the coefficient store in pinned, device-mapped host memory: the
@@ -974,6 +987,10 @@ int wv_open_stream_ex(const void *bytes, size_t n, void *device_mem, size_t devi
     *out = s;
     return WV_OK;
 }
+
+}  // namespace wv
+
+extern "C" {
 
 void wv_debug_fail_device_allocs(int n) { g_fail_allocs.store(n > 0 ? n : 0); }
 

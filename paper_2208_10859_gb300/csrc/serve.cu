@@ -141,7 +141,7 @@ int make_resident(wv_server *sv, int id, cudaStream_t cs) {
         }
     }
     wv_stream *s = nullptr;
-    const int rc = wv_open_stream(S.host, S.n, nullptr, 0, cs, &s);
+    const int rc = wv::open_stream(S.host, S.n, nullptr, 0, cs, 0, wv::kServeSets, &s);
     if (rc != WV_OK) return rc;
     // the upload is complete; later calls on the stream object (close) must
     // not name a slot's CUDA stream, which the server may destroy first
@@ -374,7 +374,7 @@ int wv_server_add_stream(wv_server *sv, const void *bytes, size_t n, int *stream
     if (!sv || !bytes || !stream_id) return WV_ERR_ARG;
     size_t need = 0;
     wv_stream_desc d;
-    const int rc = wv_stream_query(bytes, n, &d, &need);
+    const int rc = wv::query_stream(bytes, n, 0, wv::kServeSets, &d, &need);
     if (rc != WV_OK) return rc;
     SvStream S;
     if (cudaHostAlloc((void **)&S.host, n, cudaHostAllocDefault) != cudaSuccess) {

@@ -267,6 +267,11 @@ cudaError_t paper_transcode(const void *bytes, size_t n, const PaperInfo &info, 
                             cudaStream_t cs);
 
 // host helpers (api.cu)
+// wv_stream_query_ex and wv_open_stream_ex with at most max_sets buffer sets
+// (ViewSet) in the stream's device memory.
+int query_stream(const void *bytes, size_t n, int flags, int max_sets, wv_stream_desc *desc, size_t *device_bytes);
+int open_stream(const void *bytes, size_t n, void *device_mem, size_t device_bytes, void *cuda_stream, int flags,
+                int max_sets, wv_stream **out);
 int decode_region(wv_stream *s, int frame, float yaw, float pitch, float fov, int out_w, int out_h,
                   int eye = 0);
 int build_geom(const wv_stream_desc &d, Geom *g, int tile = kTile, int ctile = kCoarseTile);
@@ -400,6 +405,12 @@ namespace wv {
 // (With three internal streams shared by two sets, the coarse passes of
 // consecutive viewports ran one after the other: 143, 213, 174, 957 us.)
 constexpr int kViewSets = 4, kViewSetsLarge = 3;
+// A server decodes through batches, which have planes of their own: its
+// streams take no more than the two sets that cache budgets have been set
+// for.  (With three or four, a 4096^2 4:2:0 stream took 126 MB beside its
+// payload instead of 63, one of 8192^2 377 instead of 252, and a budget held
+// as many fewer streams.)
+constexpr int kServeSets = 2;
 struct ViewSet {
     uint32_t *tiles = nullptr, *ctiles = nullptr;        // tile lists
     uint32_t *tile_gen = nullptr, *ctile_gen = nullptr;  // stamps
