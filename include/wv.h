@@ -315,6 +315,10 @@ int wv_batch_set_wait_limit(wv_batch *b, int polls);
  * were out of memory; the calls then return WV_ERR_OOM.  n = 0 clears it. */
 void wv_debug_fail_device_allocs(int n);
 
+/* Test hook: the internal CUDA streams of closed wv_streams kept for new ones
+ * on the device (at most 16 while any wv_stream is open there, else none). */
+int wv_debug_idle_streams(int device);
+
 /* on = 1: run batches as direct launches with CUDA events between the steps
  * (wv_batch_stats reports per-step times, wv_batch_completion_ms the time
  * each request completed); on = 0: CUDA graph (default). */

@@ -264,15 +264,20 @@ int eye_view(const Geom &g, int eye, int *row0, int *rows) {
 
 // Internal streams and their events, handed from closed streams to new ones
 // (making them took 60 us of a new stream's first decode).  At most kLanesKept
-// idle ones per device; nothing in flight uses an idle one.
+// idle ones per device while a wv_stream is open there, none once the last one
+// is closed; nothing in flight uses an idle one.
 struct Lane {
     cudaStream_t st = nullptr;
     cudaEvent_t fine = nullptr, free = nullptr;
 };
 constexpr size_t kLanesKept = 16;
+struct DeviceLanes {
+    int open = 0;   // open wv_streams of the device
+    std::vector<Lane> idle;
+};
 std::mutex g_lane_mutex;
-std::map<int, std::vector<Lane>> &idle_lanes() {
-    static auto *m = new std::map<int, std::vector<Lane>>();   // outlives every stream
+std::map<int, DeviceLanes> &device_lanes() {
+    static auto *m = new std::map<int, DeviceLanes>();   // outlives every stream
     return *m;
 }
 
@@ -282,11 +287,27 @@ void destroy_lane(const Lane &l) {
         if (e) cudaEventDestroy(e);
 }
 
+// A stream of the device was opened, or closed (its lanes already given back).
+void count_open(int device) {
+    std::lock_guard<std::mutex> lock(g_lane_mutex);
+    DeviceLanes &D = device_lanes()[device];
+    D.idle.reserve(kLanesKept);   // give_lane never allocates
+    D.open += 1;
+}
+void count_closed(int device) {
+    std::vector<Lane> last;
+    {
+        std::lock_guard<std::mutex> lock(g_lane_mutex);
+        DeviceLanes &D = device_lanes()[device];
+        if (--D.open == 0) last.swap(D.idle);
+    }
+    for (const Lane &l : last) destroy_lane(l);
+}
+
 cudaError_t take_lane(int device, Lane *l) {
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
-        std::vector<Lane> &v = idle_lanes()[device];
-        v.reserve(kLanesKept);   // give_lane never allocates
+        std::vector<Lane> &v = device_lanes()[device].idle;
         if (!v.empty()) {
             *l = v.back();
             v.pop_back();
@@ -304,13 +325,19 @@ cudaError_t take_lane(int device, Lane *l) {
 void give_lane(int device, const Lane &l) {
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
-        std::vector<Lane> &v = idle_lanes()[device];
+        std::vector<Lane> &v = device_lanes()[device].idle;
         if (v.size() < kLanesKept) {
             v.push_back(l);
             return;
         }
     }
     destroy_lane(l);
+}
+
+int idle_lanes(int device) {
+    std::lock_guard<std::mutex> lock(g_lane_mutex);
+    const auto it = device_lanes().find(device);
+    return it == device_lanes().end() ? 0 : (int)it->second.idle.size();
 }
 
 // The internal stream and events of set k (when it is first used).  The set's
@@ -922,6 +949,7 @@ int open_stream(const void *bytes, size_t n, void *device_mem, size_t device_byt
         s->owns = true;
     }
     s->dbytes = L.total;
+    count_open(s->device);   // from here on the stream ends in wv_close_stream
     char *base = (char *)s->dmem;
     if (!host_payload) s->payload = (int16_t *)(base + L.payload);
     s->table = (int32_t *)(base + L.table);
@@ -994,6 +1022,8 @@ extern "C" {
 
 void wv_debug_fail_device_allocs(int n) { g_fail_allocs.store(n > 0 ? n : 0); }
 
+int wv_debug_idle_streams(int device) { return idle_lanes(device); }
+
 int wv_set_cuda_stream(wv_stream *s, void *cuda_stream) {
     if (!s) return WV_ERR_ARG;
     s->cs = (cudaStream_t)cuda_stream;
@@ -1004,6 +1034,7 @@ void wv_close_stream(wv_stream *s) {
     if (!s) return;
     cudaStreamSynchronize(s->cs);
     for (int k = 0; k < kViewSets; ++k) release_set(s, k);
+    count_closed(s->device);
     if (s->host_payload) cudaFreeHost(s->host_payload);
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     if (s->owns && s->dmem) cudaFree(s->dmem);

@@ -171,6 +171,7 @@ def _lib():
             "wv_batch_set_wait_limit": (c_int, [vp, c_int]),
             "wv_batch_set_strips": (c_int, [vp, c_int]),
             "wv_debug_fail_device_allocs": (None, [c_int]),
+            "wv_debug_idle_streams": (c_int, [c_int]),
             "wv_batch_set_tile_shape": (c_int, [vp, c_int, c_int, c_int, c_int, c_int, c_int, c_int]),
             "wv_batch_tile_shape": (c_int, [vp, c_int, c_int, c_int, c_int, ctypes.POINTER(c_int),
                                             ctypes.POINTER(c_int), ctypes.POINTER(c_int)]),
@@ -208,7 +209,7 @@ def exported_symbols() -> list[str]:
             "wv_batch_create", "wv_batch_close", "wv_batch_decode", "wv_batch_set_cuda_stream",
             "wv_batch_device_bytes", "wv_batch_sync_status", "wv_batch_stats", "wv_batch_set_timing",
             "wv_batch_set_sharing", "wv_batch_set_wait_limit", "wv_debug_fail_device_allocs",
-            "wv_batch_set_tile_shape", "wv_batch_tile_shape", "wv_batch_autotune", "wv_batch_completion_ms",
+            "wv_debug_idle_streams", "wv_batch_set_tile_shape", "wv_batch_tile_shape", "wv_batch_autotune", "wv_batch_completion_ms",
             "wv_batch_set_memory_limit", "wv_batch_set_strips"]
 
 
