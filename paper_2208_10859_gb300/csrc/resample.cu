@@ -278,6 +278,13 @@ __device__ __forceinline__ int blend_rows(int top, int bot, int fy) {
 // 4-sample groups.
 enum Chroma { kGrey = 0, kPlanar = 1, kGroups = 2 };
 
+// WV_CHECKED builds: the bytes [first, end) that one tap set loads, inside
+// the plane's n; a pixel whose taps are not is kNoSample.
+__device__ __forceinline__ bool words_in(long long first, long long end, long long n, int *err) {
+    return !kChecked || (checked_in(first, n, err) && checked_in(end - 1, n, err));
+}
+constexpr uint32_t kNoSample = 0xff000000u;
+
 // One pixel at luma position (u, w) at least two pixels inside the plane
 // (its chroma taps then lie inside theirs).
 template <int CH, bool C420>
@@ -288,7 +295,9 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
     // 8-byte aligned, rows whole groups of 8), the next word only where they
     // straddle: fewer L1 wavefronts than two byte loads
     const unsigned k = (unsigned)(X >> 8) & 7u;
-    const uint8_t *p = a.plane[0] + (unsigned)((Y >> 8) * (int)W + (X >> 8)) - k;
+    const unsigned o = (unsigned)((Y >> 8) * (int)W + (X >> 8)) - k;
+    if (!words_in(o, (long long)o + W + (k == 7 ? 12 : 8), (long long)W * a.h[0], a.err)) return kNoSample;
+    const uint8_t *p = a.plane[0] + o;
     const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p)), b = __ldg(reinterpret_cast<const uint2 *>(p + W));
     uint32_t tn = t.y, bn = b.y;
     if (k == 7) {
@@ -311,7 +320,9 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
         int cb, cr;
         if constexpr (CH == kGroups) {
             // rows are whole groups: the next row is 2 Wc bytes on
-            const uint8_t *g0 = a.plane[1] + 8u * (e >> 2);
+            const unsigned g = 8u * (e >> 2);
+            if (!words_in(g, (long long)g + 2 * Wc + ((e & 3) == 3 ? 16 : 8), 2ll * Wc * a.h[1], a.err)) return kNoSample;
+            const uint8_t *g0 = a.plane[1] + g;
             const uint2 t0 = __ldg(reinterpret_cast<const uint2 *>(g0)), b0 = __ldg(reinterpret_cast<const uint2 *>(g0 + 2 * Wc));
             uint2 t1 = t0, b1 = b0;   // the next group, where the taps straddle
             if ((e & 3) == 3) {
@@ -327,6 +338,7 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
             cb = blend_rows(cbt, cbb, gy);
             cr = blend_rows(crt, crb, gy);
         } else {
+            if (!words_in(e, (long long)e + Wc + 2, (long long)Wc * a.h[1], a.err)) return kNoSample;
             const uint8_t *p1 = a.plane[1] + e, *p2 = a.plane[2] + e;
             const uint8_t *q1 = p1 + Wc, *q2 = p2 + Wc;
             cb = blend_rows((256 - gx) * __ldg(p1) + gx * __ldg(p1 + 1), (256 - gx) * __ldg(q1) + gx * __ldg(q1 + 1), gy);
@@ -396,13 +408,8 @@ __global__ void __launch_bounds__(256) k_resample_batch(const RequestJob *__rest
     resample_any(a, blockIdx.x, blockIdx.y);
 }
 
-// Caller-given positions, luma and chroma planes instead of RGBA, and (in
-// WV_CHECKED builds) every tap checked.
+// Caller-given positions, and luma and chroma planes instead of RGBA.
 __global__ void k_resample_general(ResampleArgs a) {
-    resample_run(a, kPx * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y * blockDim.y + threadIdx.y);
-}
-__global__ void k_resample_general_batch(const RequestJob *__restrict__ reqs) {
-    const ResampleArgs &a = reqs[blockIdx.z].rs;
     resample_run(a, kPx * (blockIdx.x * blockDim.x + threadIdx.x), blockIdx.y * blockDim.y + threadIdx.y);
 }
 
@@ -429,7 +436,7 @@ void launch_resample(const Geom &g, const View &v, uint8_t *const *recon, const 
     a.uv = uv;
     a.out = out;
     a.pitch = pitch;
-    if (uv || y_plane || kChecked) {
+    if (uv || y_plane) {
         dim3 block(32, 8);
         dim3 grid((v.out_w + 32 * kPx - 1) / (32 * kPx), (v.out_h + 7) / 8);
         k_resample_general<<<grid, block, 0, cs>>>(a);
@@ -444,12 +451,6 @@ void launch_resample(const Geom &g, const View &v, uint8_t *const *recon, const 
 }
 
 void launch_resample_batch(const RequestJob *reqs, int n, int max_w, int max_h, cudaStream_t cs) {
-    if (kChecked) {
-        dim3 block(32, 8);
-        dim3 grid((max_w + 32 * kPx - 1) / (32 * kPx), (max_h + 7) / 8, n);
-        k_resample_general_batch<<<grid, block, 0, cs>>>(reqs);
-        return;
-    }
     k_resample_batch<<<dim3((max_w + kPatchW - 1) / kPatchW, (max_h + kPatchH - 1) / kPatchH, n), 256, 0, cs>>>(reqs);
 }
 
