@@ -278,10 +278,11 @@ __device__ __forceinline__ int blend_rows(int top, int bot, int fy) {
 // 4-sample groups.
 enum Chroma { kGrey = 0, kPlanar = 1, kGroups = 2 };
 
-// WV_CHECKED builds: the bytes [first, end) that one tap set loads, inside
-// the plane's n; a pixel whose taps are not is kNoSample.
-__device__ __forceinline__ bool words_in(long long first, long long end, long long n, int *err) {
-    return !kChecked || (checked_in(first, n, err) && checked_in(end - 1, n, err));
+// WV_CHECKED builds: the `bytes` bytes from `first` that one tap set lies in,
+// inside the plane's n; a pixel whose taps are not is kNoSample.
+__device__ __forceinline__ bool bytes_in(long long first, long long bytes, long long n, int *err) {
+    if constexpr (!kChecked) return true;
+    return checked_in(first, n, err) && checked_in(first + bytes - 1, n, err);
 }
 constexpr uint32_t kNoSample = 0xff000000u;
 
@@ -295,9 +296,8 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
     // 8-byte aligned, rows whole groups of 8), the next word only where they
     // straddle: fewer L1 wavefronts than two byte loads
     const unsigned k = (unsigned)(X >> 8) & 7u;
-    const unsigned o = (unsigned)((Y >> 8) * (int)W + (X >> 8)) - k;
-    if (!words_in(o, (long long)o + W + (k == 7 ? 12 : 8), (long long)W * a.h[0], a.err)) return kNoSample;
-    const uint8_t *p = a.plane[0] + o;
+    const uint8_t *p = a.plane[0] + (unsigned)((Y >> 8) * (int)W + (X >> 8)) - k;
+    if (!bytes_in(p - a.plane[0], W + (k == 7 ? 12 : 8), (long long)W * a.h[0], a.err)) return kNoSample;
     const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p)), b = __ldg(reinterpret_cast<const uint2 *>(p + W));
     uint32_t tn = t.y, bn = b.y;
     if (k == 7) {
@@ -320,9 +320,8 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
         int cb, cr;
         if constexpr (CH == kGroups) {
             // rows are whole groups: the next row is 2 Wc bytes on
-            const unsigned g = 8u * (e >> 2);
-            if (!words_in(g, (long long)g + 2 * Wc + ((e & 3) == 3 ? 16 : 8), 2ll * Wc * a.h[1], a.err)) return kNoSample;
-            const uint8_t *g0 = a.plane[1] + g;
+            const uint8_t *g0 = a.plane[1] + 8u * (e >> 2);
+            if (!bytes_in(g0 - a.plane[1], 2 * Wc + ((e & 3) == 3 ? 16 : 8), 2ll * Wc * a.h[1], a.err)) return kNoSample;
             const uint2 t0 = __ldg(reinterpret_cast<const uint2 *>(g0)), b0 = __ldg(reinterpret_cast<const uint2 *>(g0 + 2 * Wc));
             uint2 t1 = t0, b1 = b0;   // the next group, where the taps straddle
             if ((e & 3) == 3) {
@@ -338,7 +337,7 @@ __device__ __forceinline__ uint32_t inside_px(const ResampleArgs &a, int X, int 
             cb = blend_rows(cbt, cbb, gy);
             cr = blend_rows(crt, crb, gy);
         } else {
-            if (!words_in(e, (long long)e + Wc + 2, (long long)Wc * a.h[1], a.err)) return kNoSample;
+            if (!bytes_in(e, Wc + 2, (long long)Wc * a.h[1], a.err)) return kNoSample;
             const uint8_t *p1 = a.plane[1] + e, *p2 = a.plane[2] + e;
             const uint8_t *q1 = p1 + Wc, *q2 = p2 + Wc;
             cb = blend_rows((256 - gx) * __ldg(p1) + gx * __ldg(p1 + 1), (256 - gx) * __ldg(q1) + gx * __ldg(q1 + 1), gy);
