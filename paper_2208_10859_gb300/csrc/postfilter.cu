@@ -115,6 +115,7 @@ constexpr int kBBlock = 4 * 256;        // 32 output channels x 16 K
 constexpr int kBMidF = 6 * kSeq * kBBlock;
 constexpr int kBLastF = 6 * kSeq * (kBBlock / 2);
 constexpr int kA0 = 128 * 32;           // stage 0's operand: 128 pixels x 16 taps
+constexpr int kWaitRound = 1 << 14, kWaitRounds = 64;   // polls between looks at the stop flag; default limit
 constexpr int kNetRing = 4 * kRings * kSlot;
 constexpr int kNetSmem = kNetRing + 3 * kBMidF + kBLastF + kBIn1 + 2 * kA0;
 
@@ -136,6 +137,7 @@ struct NetArgs {
     uint8_t *rgba;
     size_t pitch;
     int *err;
+    int wait_rounds;                    // rounds of kWaitRound polls before a wait gives up
 };
 
 struct NetBars {
@@ -147,9 +149,12 @@ struct NetBars {
 
 // Waits for the phase; false (and the flag set) when the limit is reached or
 // another role has given up.
-__device__ __forceinline__ bool net_wait(uint64_t *bar, uint32_t parity, volatile int *stop) {
-    for (int k = 0; k < 64; ++k) {
-        if (umma::mbar_wait(bar, parity, 1 << 14)) return true;
+// LIMIT: the caller's limit (kernels of their own: read at run time it cost the
+// forward pass 4 %), else the default.
+template <bool LIMIT>
+__device__ __forceinline__ bool net_wait(const NetArgs &a, uint64_t *bar, uint32_t parity, volatile int *stop) {
+    for (int k = 0; k < (LIMIT ? a.wait_rounds : kWaitRounds); ++k) {
+        if (umma::mbar_wait(bar, parity, kWaitRound)) return true;
         if (*stop) return false;
     }
     *stop = 1;
@@ -157,8 +162,9 @@ __device__ __forceinline__ bool net_wait(uint64_t *bar, uint32_t parity, volatil
 }
 
 // The same for a whole warp, with one answer for all its lanes.
-__device__ __forceinline__ bool net_wait_warp(uint64_t *bar, uint32_t parity, volatile int *stop) {
-    return __all_sync(0xffffffffu, net_wait(bar, parity, stop));
+template <bool LIMIT>
+__device__ __forceinline__ bool net_wait_warp(const NetArgs &a, uint64_t *bar, uint32_t parity, volatile int *stop) {
+    return __all_sync(0xffffffffu, net_wait<LIMIT>(a, bar, parity, stop));
 }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
@@ -187,7 +193,7 @@ __device__ __forceinline__ int net_tasks(const NetArgs &a) {
 }
 
 // The warp that issues stage 0's MMAs (control flow and operands uniform).
-template <int T>
+template <int T, bool LIMIT>
 __device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, const uint8_t *sA0, NetBars *bars,
                                            uint32_t tmem, volatile int *stop) {
     const uint64_t bd = umma::desc(umma::smem_addr(sB) + 3 * kBMidF + kBLastF, 128, 256);
@@ -197,7 +203,7 @@ __device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, 
         const NetTask k = net_task(a, it);
         for (int j = 0; j < k.y1 - k.y0 + 2 * T; ++j, ++r) {
             const int b = r & 1;
-            if (!net_wait_warp(&bars->a0_full[b], (r >> 1) & 1, stop)) return;
+            if (!net_wait_warp<LIMIT>(a, &bars->a0_full[b], (r >> 1) & 1, stop)) return;
             umma::fence_after_sync();
             if (umma::elect_one()) {
                 umma::mma(tmem + acc_col(0) + 32 * b, ad + b * (kA0 >> 4), bd, umma::idesc_bf16(128, 32), false);
@@ -212,7 +218,7 @@ __device__ __forceinline__ void net_issue0(const NetArgs &a, const uint8_t *sB, 
 // NC: accumulator columns per slot).  Input row j of a task takes part in
 // the output rows j - 2 .. j (counted from the task's first), which live in
 // the slots of their index mod 3.
-template <int T, int BLK, int NC>
+template <int T, int BLK, int NC, bool LIMIT>
 __device__ __forceinline__ void net_issue(const NetArgs &a, int l, const uint8_t *rings, const uint8_t *sB,
                                           NetBars *bars, uint32_t tmem, volatile int *stop) {
     const uint64_t ad = umma::desc(umma::smem_addr(rings) + (l - 1) * kRings * kSlot, kLbo, 128);
@@ -224,9 +230,9 @@ __device__ __forceinline__ void net_issue(const NetArgs &a, int l, const uint8_t
         const int rows = k.y1 - k.y0 + 2 * (T - l + 1);
         for (int j = 0; j < rows; ++j, ++u) {
             const int b = u % kRings;
-            if (!net_wait_warp(&bars->in_full[l][b], (u / kRings) & 1, stop)) return;
+            if (!net_wait_warp<LIMIT>(a, &bars->in_full[l][b], (u / kRings) & 1, stop)) return;
             if (j == 0 || j >= 3) {   // output row j's slot is free
-                if (!net_wait_warp(&bars->drained[l], drains & 1, stop)) return;
+                if (!net_wait_warp<LIMIT>(a, &bars->drained[l], drains & 1, stop)) return;
                 ++drains;
             }
             umma::fence_after_sync();
@@ -293,7 +299,7 @@ __device__ __forceinline__ float store_last(const NetArgs &a, size_t p, float r,
 }
 
 // A stage's warpgroup (thread = pixel of the tile).  T: the last stage.
-template <bool BWD, int T>
+template <bool BWD, int T, bool LIMIT>
 __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *rings, uint8_t *sA0, const float *bias,
                                           NetBars *bars, uint32_t tmem, volatile int *stop) {
     const int px = threadIdx.x & 127, lane = threadIdx.x & 31;
@@ -375,9 +381,9 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
                 if (a.mode == kTrain) tv = __ldg(a.t + p);
             }
             if (l == 0) {
-                if (!net_wait_warp(&bars->acc0_full[outs & 1], (outs >> 1) & 1, stop)) return;
+                if (!net_wait_warp<LIMIT>(a, &bars->acc0_full[outs & 1], (outs >> 1) & 1, stop)) return;
             } else {
-                if (!net_wait_warp(&bars->acc_full[l], outs & 1, stop)) return;
+                if (!net_wait_warp<LIMIT>(a, &bars->acc_full[l], outs & 1, stop)) return;
             }
             umma::fence_after_sync();
             if (!BWD && l == 4) {
@@ -415,7 +421,7 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
             // into the next stage's ring (the last stage's rows only pass
             // through it on their way to memory)
             const int b = outs % kRings;
-            if (l < T && outs >= kRings && !net_wait_warp(&bars->in_free[l + 1][b], (outs / kRings - 1) & 1, stop)) return;
+            if (l < T && outs >= kRings && !net_wait_warp<LIMIT>(a, &bars->in_free[l + 1][b], (outs / kRings - 1) & 1, stop)) return;
             uint8_t *row = rings + (l * kRings + b) * kSlot + 16;
 #pragma unroll
             for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4 *>(row + px * 16 + c * kLbo) = o[c];
@@ -445,7 +451,7 @@ __device__ __forceinline__ void net_stage(const NetArgs &a, int l, uint8_t *ring
     }
 }
 
-template <bool BWD>
+template <bool BWD, bool LIMIT>
 __global__ void __launch_bounds__(net_threads(BWD), 1) k_net(NetArgs a) {
     constexpr int T = BWD ? 3 : 4, kNetThreads = net_threads(BWD);
     extern __shared__ __align__(128) uint8_t sm[];
@@ -505,16 +511,16 @@ __global__ void __launch_bounds__(net_threads(BWD), 1) k_net(NetArgs a) {
     const uint32_t tmem = tmem_base;
     if (warp >= 4 * (T + 1)) {
         const int l = warp - 4 * (T + 1);
-        if (l == 0) net_issue0<T>(a, sB, sA0, &bars, tmem, &stop);
-        else if (l < 4) net_issue<T, kBBlock, 32>(a, l, rings, sB, &bars, tmem, &stop);
-        else net_issue<T, kBBlock / 2, 16>(a, l, rings, sB, &bars, tmem, &stop);
+        if (l == 0) net_issue0<T, LIMIT>(a, sB, sA0, &bars, tmem, &stop);
+        else if (l < 4) net_issue<T, kBBlock, 32, LIMIT>(a, l, rings, sB, &bars, tmem, &stop);
+        else net_issue<T, kBBlock / 2, 16, LIMIT>(a, l, rings, sB, &bars, tmem, &stop);
         if (umma::elect_one()) {
             umma::commit(&bars.idle[l]);
             umma::mbar_wait(&bars.idle[l], 0);
         }
         __syncwarp();
     } else {
-        net_stage<BWD, T>(a, warp >> 2, rings, sA0, sBias[warp >> 2], &bars, tmem, &stop);
+        net_stage<BWD, T, LIMIT>(a, warp >> 2, rings, sA0, sBias[warp >> 2], &bars, tmem, &stop);
     }
     umma::fence_before_sync();
     __syncthreads();
@@ -888,6 +894,7 @@ struct wv_cnn {
     size_t cap_train = 0, cap_view = 0;
     std::vector<void *> owned_train, owned_view;
     int *err = nullptr;
+    int wait_rounds = kWaitRounds;     // of the fused kernels' bounded waits
 };
 
 namespace {
@@ -953,14 +960,20 @@ int seg_rows(int n, int h, int w, int T) {
     return seg;
 }
 
+template <bool BWD, bool LIMIT>
+cudaError_t launch_net_as(const NetArgs &a, int grid, cudaStream_t cs) {
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_net<BWD, LIMIT>), kNetSmem);
+    if (e != cudaSuccess) return e;
+    k_net<BWD, LIMIT><<<grid, net_threads(BWD), kNetSmem, cs>>>(a);
+    return cudaGetLastError();
+}
+
 template <bool BWD>
 cudaError_t launch_net(NetArgs &a, cudaStream_t cs) {
-    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(k_net<BWD>), kNetSmem);
-    if (e != cudaSuccess) return e;
     a.seg = seg_rows(a.n, a.h, a.w, BWD ? 3 : 4);
     const long long tasks = (long long)a.n * ((a.w + kTileOut - 1) / kTileOut) * ((a.h + a.seg - 1) / a.seg);
-    k_net<BWD><<<(int)std::min<long long>(tasks, sm_count()), net_threads(BWD), kNetSmem, cs>>>(a);
-    return cudaGetLastError();
+    const int grid = (int)std::min<long long>(tasks, sm_count());
+    return a.wait_rounds == kWaitRounds ? launch_net_as<BWD, false>(a, grid, cs) : launch_net_as<BWD, true>(a, grid, cs);
 }
 
 cudaError_t launch_wgrad_mid(const WgradArgs &a, cudaStream_t cs) {
@@ -994,6 +1007,7 @@ cudaError_t forward(wv_cnn *c, const float *x, int n, int h, int w, NetArgs &a, 
     a.h = h;
     a.w = w;
     a.err = c->err;
+    a.wait_rounds = c->wait_rounds;
     for (int l = 0; l < kStages; ++l) {
         a.pack[l] = c->pack + packs[l];
         a.bias[l] = c->params + off_b(l);
@@ -1025,6 +1039,7 @@ cudaError_t forward_backward(wv_cnn *c, const float *x, const float *t, int n, i
     a.h = h;
     a.w = w;
     a.err = c->err;
+    a.wait_rounds = c->wait_rounds;
     for (int s = 0; s < 4; ++s) {
         a.pack[s] = c->pack + packs[s];
         a.gate[s] = c->act[3 - s];
@@ -1210,6 +1225,12 @@ int wv_cnn_train_step(wv_cnn *c, const float *x_dev, const float *t_dev, int n, 
             return WV_ERR_CUDA;
         *loss_host = loss / (float)((double)n * h * w);
     }
+    return WV_OK;
+}
+
+int wv_cnn_set_wait_limit(wv_cnn *c, int polls) {
+    if (!c || polls < 0) return WV_ERR_ARG;
+    c->wait_rounds = std::min(polls / kWaitRound + (polls % kWaitRound != 0), kWaitRounds);
     return WV_OK;
 }
 

@@ -143,6 +143,7 @@ def _lib():
             "wv_cnn_gradients": (c_int, [vp, vp, vp, c_int, c_int, c_int, vp, ctypes.POINTER(fl), vp]),
             "wv_cnn_train_step": (c_int, [vp, vp, vp, c_int, c_int, c_int, fl, ctypes.POINTER(fl), vp]),
             "wv_cnn_sync_status": (c_int, [vp]),
+            "wv_cnn_set_wait_limit": (c_int, [vp, c_int]),
             "wv_decode_viewport_filtered": (c_int, [vp, c_int, fl, fl, fl, vp, ctypes.POINTER(Image)]),
             "wv_server_create": (c_int, [ctypes.POINTER(ServerConfig), ctypes.POINTER(vp)]),
             "wv_server_add_stream": (c_int, [vp, vp, c_size, ctypes.POINTER(c_int)]),
@@ -202,6 +203,7 @@ def exported_symbols() -> list[str]:
             "wv_cnn_param_count", "wv_cnn_create", "wv_cnn_close", "wv_cnn_get_params", "wv_cnn_set_params",
             "wv_cnn_get_state", "wv_cnn_set_state",
             "wv_cnn_forward", "wv_cnn_gradients", "wv_cnn_train_step", "wv_cnn_sync_status",
+            "wv_cnn_set_wait_limit",
             "wv_decode_viewport_filtered",
             "wv_server_create", "wv_server_add_stream", "wv_server_submit", "wv_server_poll",
             "wv_server_wait", "wv_server_drain", "wv_server_get_stats", "wv_server_latencies",
@@ -721,6 +723,10 @@ class CNN:
                                         ctypes.byref(loss) if want_loss else None,
                                         ctypes.c_void_p(_cuda_stream_handle(stream))), "wv_cnn_train_step")
         return float(loss.value) if want_loss else None
+
+    def set_wait_limit(self, polls: int) -> None:
+        """Polls of the fused kernels' bounded waits before they give up."""
+        _check(_lib().wv_cnn_set_wait_limit(self.handle, int(polls)), "wv_cnn_set_wait_limit")
 
     def sync_status(self) -> int:
         return _lib().wv_cnn_sync_status(self.handle)
