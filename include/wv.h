@@ -492,11 +492,12 @@ int wv_cnn_gradients(wv_cnn *c, const float *x_dev, const float *t_dev, int n, i
 int wv_cnn_train_step(wv_cnn *c, const float *x_dev, const float *t_dev, int n, int h, int w, float lr,
                       float *loss_host, void *cuda_stream);
 
-/* Polls of the fused kernels' bounded waits (one stage waiting for another)
- * before they give up, record WV_ERR_TIMEOUT and end, leaving the output
- * undefined.  Default and maximum 2^20, rounded up to a multiple of 2^14;
- * polls = 0 makes every wait give up at once -- the failure path, exercised
- * without a GPU fault.  Takes effect from the next call. */
+/* Polls of the bounded waits of the network's tensor-core kernels (one stage
+ * waiting for another, or for its products) before they give up, record
+ * WV_ERR_TIMEOUT and end, leaving their output undefined.  Default and
+ * maximum 2^20, rounded up to a multiple of 2^14; polls = 0 makes every wait
+ * give up at once -- the failure path, exercised without a GPU fault.  Takes
+ * effect from the next call. */
 int wv_cnn_set_wait_limit(wv_cnn *c, int polls);
 
 /* Synchronise the device and read the network's error word (WV_ERR_TIMEOUT:

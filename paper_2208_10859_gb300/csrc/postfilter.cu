@@ -570,6 +570,7 @@ struct WgradArgs {
     float *dW[kMidLayers], *db[kMidLayers];   // dW 16-byte aligned
     int layers, n, h, w;
     int *err;
+    int polls;   // of a wait for the MMAs before it gives up
 };
 
 __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(WgradArgs args) {
@@ -619,12 +620,13 @@ __global__ void __launch_bounds__(kWThreads, 2) k_wgrad_mid(WgradArgs args) {
     bool first = true, ok = true;
     float bsum[8] = {};   // channels 8 q ..
     auto wait_mma = [&]() {
-        const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase));
-        phase ^= 1;
+        const bool got = __syncthreads_and(umma::mbar_wait(&mbar, phase, args.polls));
         if (!got) {
             ok = false;
             if (tid == 0) record_error(err, WV_ERR_TIMEOUT);
+            umma::mbar_wait(&mbar, phase);   // no MMA in flight when the CTA ends
         }
+        phase ^= 1;
     };
     for (int it = cta; it < total; it += ctas) {
         if (!first) wait_mma();
@@ -894,7 +896,7 @@ struct wv_cnn {
     size_t cap_train = 0, cap_view = 0;
     std::vector<void *> owned_train, owned_view;
     int *err = nullptr;
-    int wait_rounds = kWaitRounds;     // of the fused kernels' bounded waits
+    int wait_rounds = kWaitRounds;     // limit of the tensor-core kernels' bounded waits
 };
 
 namespace {
@@ -1055,6 +1057,7 @@ cudaError_t forward_backward(wv_cnn *c, const float *x, const float *t, int n, i
     m.h = h;
     m.w = w;
     m.err = c->err;
+    m.polls = c->wait_rounds * kWaitRound;
     for (int l = 1; l <= kMidLayers; ++l) {
         m.act[l - 1] = c->act[l - 1];
         m.dz[l - 1] = c->g[l];

@@ -725,7 +725,7 @@ class CNN:
         return float(loss.value) if want_loss else None
 
     def set_wait_limit(self, polls: int) -> None:
-        """Polls of the fused kernels' bounded waits before they give up."""
+        """Polls of the tensor-core kernels' bounded waits before they give up."""
         _check(_lib().wv_cnn_set_wait_limit(self.handle, int(polls)), "wv_cnn_set_wait_limit")
 
     def sync_status(self) -> int:

@@ -46,3 +46,24 @@ def test_waits_that_run_out_are_reported():
         net.set_wait_limit(-1)
     assert s.sync_status() == 0
     net.close()
+
+
+def test_gradients_whose_waits_run_out():
+    """The weight-gradient kernel gives up too, and waits for its products in
+    flight before it ends; the next call's gradients are those of an untouched
+    network (their sums' order varies, so to rounding)."""
+    from paper_2208_10859_gb300 import wv
+    net = wv.CNN(seed=4)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    x, t = (torch.rand((4, 130, 300), generator=g, device="cuda") for _ in range(2))
+    loss, grads = net.gradients(x, t)
+    for _ in range(2):
+        net.set_wait_limit(0)
+        net.gradients(x, t)
+        assert net.sync_status() == WV_ERR_TIMEOUT
+        net.set_wait_limit(1 << 20)
+        loss2, grads2 = net.gradients(x, t)
+        assert net.sync_status() == 0
+        assert abs(loss2 - loss) <= 1e-5 * loss
+        assert abs(grads2 - grads).max() <= 1e-4 * abs(grads).max()
+    net.close()
