@@ -743,7 +743,7 @@ def lossless_leg(dev, stream):
     return {"workload": "512x512 grey, 3-level LeGall 5/3 integer, step 1 (lossless), whole-plane decode",
             "gpu_ms_per_frame": gpu_ms, "oracle_ms_per_frame_1_thread": oracle_ms,
             "bit_exact_gpu": exact and ok, "bit_exact_oracle": bool(np.array_equal(u8, img)),
-            "gpu_launches_per_frame": 4}
+            "gpu_launches_per_frame": 2}
 
 
 def run_reference(args):

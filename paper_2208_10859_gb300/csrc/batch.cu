@@ -78,7 +78,7 @@ struct Surface {
 constexpr size_t kWaitWord = 64;
 
 // A wave: surfaces [s0, s1) and the rows [r0, r1) of the request table (the
-// table lists requests by wave, in caller order inside a wave).
+// table lists requests by wave and decode class, in caller order inside a class).
 struct Wave {
     int s0, s1, r0, r1;
     size_t ctr;            // its counters (kBatchCtr + 2 (s1 - s0) ints)

@@ -144,7 +144,7 @@ __global__ void k_footprint(View v, Frustum f, Geom g, uint8_t *__restrict__ mas
                             uint32_t gen, int *counters) {
     const int cx = blockIdx.x * blockDim.x + threadIdx.x;
     const int cy = blockIdx.y * blockDim.y + threadIdx.y;
-    if (cx == 0 && cy == 0) counters[0] = counters[1] = counters[2] = 0;   // tile counts of this viewport
+    if (cx == 0 && cy == 0) counters[0] = counters[1] = 0;   // tile counts of this viewport
     if (cx >= g.cells_x || cy >= g.cells_y) return;
     const bool hit = cell_needed_eye(v, f, g.p[0].w, cx, cy);
     if (mask) mask[cy * g.cells_x + cx] = hit ? 1 : 0;
@@ -260,13 +260,9 @@ __global__ void k_select_batch(const SurfaceJob *__restrict__ surfs, BatchLists 
     append2(sel && is_coarse, e, lists.coarse[c], &ctr[4 * c + 1]);
 }
 
-__global__ void k_all_tiles(int plane, int tiles_x, int tiles_y, uint32_t *tiles,
-                            int *count, int *work) {
+__global__ void k_all_tiles(int plane, int tiles_x, int tiles_y, uint32_t *tiles, int *count) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0) {
-        *count = tiles_x * tiles_y;
-        if (work) *work = 0;
-    }
+    if (t == 0) *count = tiles_x * tiles_y;
     if (t >= tiles_x * tiles_y) return;
     tiles[t] = ((uint32_t)plane << 28) | ((uint32_t)(t / tiles_x) << 14) | (uint32_t)(t % tiles_x);
 }
@@ -317,14 +313,14 @@ void launch_all_tiles(const Geom &g, int plane, uint32_t *tiles, int *counters,
                       cudaStream_t cs) {
     const int n = g.p[plane].tiles_x * g.p[plane].tiles_y;
     k_all_tiles<<<(n + 255) / 256, 256, 0, cs>>>(plane, g.p[plane].tiles_x, g.p[plane].tiles_y,
-                                                 tiles, &counters[0], &counters[2]);
+                                                 tiles, &counters[0]);
 }
 
 void launch_all_ctiles(const Geom &g, int plane, uint32_t *ctiles, int *counters,
                        cudaStream_t cs) {
     const int n = g.p[plane].ctiles_x * g.p[plane].ctiles_y;
     k_all_tiles<<<(n + 255) / 256 > 0 ? (n + 255) / 256 : 1, 256, 0, cs>>>(
-        plane, g.p[plane].ctiles_x, g.p[plane].ctiles_y, ctiles, &counters[1], nullptr);
+        plane, g.p[plane].ctiles_x, g.p[plane].ctiles_y, ctiles, &counters[1]);
 }
 
 void launch_project(const View &v, float *uv, cudaStream_t cs) {

@@ -158,12 +158,5 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
     asm volatile("{\n.reg .b64 s;\nmbarrier.arrive.shared::cta.b64 s, [%0];\n}" ::"r"(smem_addr(mbar)) : "memory");
 }
 
-// Byte offset of element (r, k) in a K-major, no-swizzle tile of R rows and
-// 16 K elements (one MMA K-step): core matrix (r / 8, k / 8) at
-// (r / 8) * 256 + (k / 8) * 128 (LBO 128, SBO 256).
-__host__ __device__ __forceinline__ int kstep_offset(int r, int k) {
-    return (r >> 3) * 256 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
-
 }  // namespace umma
 }  // namespace wv

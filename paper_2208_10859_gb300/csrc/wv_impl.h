@@ -459,7 +459,6 @@ struct wv_stream {
     std::vector<cudaEvent_t> ev_pool;
     std::vector<int> ev_kind;
     size_t ev_used = 0;
-    int last_tiles = 0;
 };
 
 #ifdef __CUDACC__
