@@ -31,7 +31,11 @@ SAN_FLAGS = ["-Xcompiler=-fsanitize=address", "-Xcompiler=-fsanitize=undefined",
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-O2",
+# -no-compress: nvcc compresses device code above a size of its own, and the
+# driver unpacks a whole translation unit at a process's first use of one of
+# its kernels: 13 ms in the first viewport (strip.cu), 20 in the first open
+# (ifwt.cu); stored as it is, 1.8 and 2.5.  The library is 36 MB instead of 10.
+NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-no-compress", "-Xcompiler", "-fPIC,-O2",
               "--expt-relaxed-constexpr", "-I", INCLUDE]
 
 

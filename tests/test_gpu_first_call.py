@@ -1,0 +1,51 @@
+"""The first calls of a process: the kernels' code is loaded at their first use,
+which must not cost a player its first frames.  Opening a small stream and
+decoding its first viewport take 2.5 and 1.8 ms in a fresh process; with the
+device code compressed in the library they took 20 and 13.  The bounds lie at
+twice the former (best of three processes)."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+SCRIPT = r'''
+import sys, time
+sys.path.insert(0, ROOT)
+import torch
+out = torch.zeros((120, 160, 4), dtype=torch.uint8, device="cuda")
+data = sys.stdin.buffer.read()
+from paper_2208_10859_gb300 import wv
+wv._lib()
+torch.empty(1 << 24, dtype=torch.uint8, device="cuda")     # PyTorch's pool holds the stream's memory
+torch.cuda.synchronize()
+t = [time.perf_counter()]
+s = wv.Stream(data)
+torch.cuda.synchronize()
+t.append(time.perf_counter())
+s.decode_viewport(0, 0.3, 0.1, 1.5, out)
+torch.cuda.synchronize()
+t.append(time.perf_counter())
+assert s.sync_status() == 0 and float(out.float().std()) > 5
+print(1e3 * (t[1] - t[0]), 1e3 * (t[2] - t[1]))
+'''
+
+
+def test_first_open_and_first_viewport_of_a_process():
+    data = H.case("yuv97")[2]
+    runs = []
+    for _ in range(3):
+        r = subprocess.run([sys.executable, "-c", f"ROOT = {ROOT!r}\n" + SCRIPT], input=data, cwd=HERE,
+                           capture_output=True, timeout=600)
+        assert r.returncode == 0, r.stderr[-4000:].decode()
+        runs.append([float(v) for v in r.stdout.split()])
+    opened, viewport = (min(c) for c in zip(*runs))
+    assert opened < 5.0, runs
+    assert viewport < 4.0, runs
