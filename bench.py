@@ -353,8 +353,9 @@ def batched_leg(args, dev, frames8k, stream):
                             "frac": dec_gbs / peak,
                             "algorithmic_bytes": alg_total,
                             "bytes_note": "coefficient cone (with foveation) + decoded region, exact on every 8th request, scaled to 256"},
-        "gpu_launches_per_batch": 3 + len({(r.stream.desc["wavelet"], r.stream.desc["tlevels"], r.fovea)
-                                           for r in reqs}),
+        # per wave: footprint, selection, and coarse tiles, strips and resampling of each decode class
+        "gpu_launches_per_batch": info["waves"] * (2 + 3 * len({(r.stream.desc["wavelet"], r.stream.desc["tlevels"],
+                                                                 r.fovea) for r in reqs})),
     }
 
 

@@ -261,10 +261,11 @@ void wv_batch_close(wv_batch *b);
  * tables from pinned host memory and the clearing of the counters, then per
  * wave of decode targets (1) clearing of the wave's stamps, (2) the
  * footprint of every request of the wave, (3) the tile lists of every decode
- * target of the wave, (4) per decode class (wavelet and 1 + tlevels
- * coefficient frames) one persistent tile-decode launch over every coarse
- * tile (levels L..3), then every output tile (levels 2..1) of its targets,
- * and (5) the reprojection of every request of the wave.  Unfoveated
+ * target of the wave, then, as a branch of the graph for each decode class
+ * (wavelet, foveation and 1 + tlevels coefficient frames), (4) one persistent
+ * tile-decode launch over every coarse tile (levels L..3) and square output
+ * tile of its targets, one launch over their strips (levels 2..1), and (5) the
+ * reprojection of the class's requests.  Unfoveated
  * requests of the same stream and frame share one decode target, so a tile
  * several of them need is decoded once; a foveated request (Sec. 3.7) has
  * its own.  Targets are grouped into waves in request order.  The

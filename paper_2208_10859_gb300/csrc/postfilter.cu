@@ -99,9 +99,12 @@ enum Mode { kTrain = 0, kOut = 1, kRgba = 2 };   // the last layer's epilogue
 // mbarrier wait with a limit; one that gives up sets a flag that ends all
 // roles.
 //
-// Bound: the tensor pipe (an MMA takes about one cycle per accumulator column
-// here, 290 us of a 2160^2 plane's 306).  Layer by layer, 2.4 GB of
-// activations through HBM, the plane took 887 us.  Training adds 512 bytes a
+// Bound: the MMAs, which take about one cycle per accumulator column here (by
+// count of columns, 290 us of a 2160^2 plane's 306), and that is half the
+// tensor pipe's rate: its counter shows 43 % active, with 54 % of the issue
+// slots and 38 % of the shared-memory wavefronts used, and DRAM idle.  Why an
+// MMA of N = 96 does not take half the cycles is not known.  Layer by layer,
+// 2.4 GB of activations through HBM, the plane took 887 us.  Training adds 512 bytes a
 // pixel of activations and gradients kept: 144 us forward and 155 us for the
 // input gradients of 16 x 256^2 pixels (270 and 230 layer by layer).
 
@@ -543,9 +546,11 @@ __global__ void __launch_bounds__(net_threads(BWD), 1) k_net(NetArgs a) {
 // The bias gradient is summed from the dz rows in shared memory meanwhile.
 //
 // Bound: the MMAs' reads of A (4 KB per 16 pixels and dx) and the 128 bytes
-// per pixel from HBM, about 20 us each for 16 x 256^2 pixels; two CTAs per SM
-// so that one's loads run under the other's MMAs (one CTA with two operand
-// buffers: 88 us, too few warps issuing loads).  One
+// per pixel from HBM, about 20 us each for 16 x 256^2 pixels of a layer, and
+// the waits of a CTA between its loads and its MMAs; two CTAs per SM so that
+// one's loads run under the other's MMAs (one CTA with two operand buffers:
+// 88 us, too few warps issuing loads).  Counters of the three layers' launch:
+// tensor pipe 18 % active, DRAM 27 %, warps stalled on their loads.  One
 // layer alone takes 70 us (with both operands transposed through shared memory
 // by the threads 434), the three of a step in one launch 190: a third of the
 // CTAs' fills, drains and gradient additions, which go out four floats at a

@@ -215,7 +215,8 @@ __device__ __forceinline__ void resample_run(const ResampleArgs &a, int i, int j
 //     the second word is loaded by the lanes that need it only (24 foveated
 //     viewports 1441 -> 1431 us, 12 of shared frames 390 -> 383).
 // One row of pixel pairs per warp took 284 instructions a pixel and 9.8 L1
-// wavefronts a load, 53 us per 2160^2 viewport; this takes 30 (24 in a launch).
+// wavefronts a load, 53 us per 2160^2 viewport; this takes 187 and 5.6, 38 us
+// alone and 30 with 24 viewports in a launch (80 % of the issue slots).
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }

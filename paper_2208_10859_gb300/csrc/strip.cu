@@ -810,8 +810,9 @@ __device__ __forceinline__ void strip_tile(const TileArgs &a, uint32_t e, float 
     }
 }
 
-// One warp per CTA.  A launch has room for 12 strips per SM (168 registers a
-// thread) and lasts as long as its slowest tile, so warps that find no tile
+// One warp per CTA.  A launch has room for 12 strips per SM (at most 168
+// registers a thread; the 9/7 pair kernel takes 154) and lasts as long as its
+// slowest tile, so warps that find no tile
 // or finish early must give their registers and shared memory back at once:
 // the coarse pass of the next viewport and the resampling of the previous one
 // run beside this kernel on what is free.  With four warps per CTA the slots
@@ -982,7 +983,12 @@ cudaError_t launch_decode_strips(const Geom &g, const int16_t *payload, const in
         // tile of h rows takes h / 4 + 7 iterations, and twice the warps on
         // an SM do not double an iteration's time), else the default.  The
         // planes of a 2048 x 1024 4:2:0 frame: 64 rows, with tile lists 255
-        // us; this 138, with coarse tiles of 32 115.
+        // us; this 138, with coarse tiles of 32 115.  One 9/7 plane as bytes
+        // in 16, 32, 64 rows, us: 512^2 25, 34, 52; 2048 x 1024 34, 42, 58;
+        // 2880 x 1440 37, 44, 59; 2048^2 38, 49, 63; 4096 x 2048 52, 43, 59;
+        // 4096^2 89, 86, 76; 8192 x 4096 165, 135, 155; 8192^2 280, 232, 221.
+        // (So 12 strips per SM would be the better line for frames between
+        // 912 and 1824 strips of a height; above that the best varies.)
         const PlaneGeom &pg = g.p[all_plane];
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);

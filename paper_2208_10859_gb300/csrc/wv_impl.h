@@ -289,7 +289,9 @@ bool strip_eligible(const wv_stream_desc &d, uint64_t n_payload);
 // strip of h rows takes h / 4 + 7 iterations of one warp), so while a
 // viewport's tiles do not fill the chip, lower tiles finish sooner; they redo
 // more warm-up rows, which costs once the chip is full.  The line is where a
-// viewport's 32-row strips are eight warps per SM (152 SMs).  Default against
+// viewport's 32-row strips are eight warps per SM.  The count of SMs is this
+// chip's (152), not the device's: the line decides the size of a stream's
+// device memory, which wv_stream_query gives without a device.  Default against
 // finer tiles: 4 viewports of 2880 x 1440 229 -> 145 us, of 4096 x 2048 per eye
 // 272 -> 214 us, of 6144 x 3072 186 -> 174 us; 8 of 8192^2 (above the line)
 // 961 -> 1031 us.  Halves everywhere below the line: 6144 x 3072 174 -> 186 us.
@@ -401,7 +403,8 @@ namespace wv {
 // bound by the length of that chain, not by its work, and take four sets,
 // larger ones three.  Four viewports (eight of 8192^2) with two sets, three,
 // four: 2880 x 1440 126, 116, 95 us; 4096^2 stereo 185, 178, 156; 6144 x 3072
-// 165, 159, 143; 8192^2 913, 866, 866.  Six for the small ones gave nothing.
+// 165, 159, 143; 8192^2 913, 866, 866 (with the resampler of the time; 706 with
+// three sets and the present one).  Six for the small ones gave nothing.
 // (With three internal streams shared by two sets, the coarse passes of
 // consecutive viewports ran one after the other: 143, 213, 174, 957 us.)
 constexpr int kViewSets = 4, kViewSetsLarge = 3;
