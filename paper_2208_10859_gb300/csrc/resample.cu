@@ -233,15 +233,15 @@ __device__ __forceinline__ float2 atan2_pair(float2 y, float2 x) {
     if (!(mx0 > 0.0f)) t.x = 0.0f;
     if (!(mx1 > 0.0f)) t.y = 0.0f;
     const float2 u = __fmul2_rn(t, t);
-    float2 p = f2(-0.0017539301188662648f);
-    p = __ffma2_rn(p, u, f2(0.010726944543421268f));
-    p = __ffma2_rn(p, u, f2(-0.030804596841335297f));
-    p = __ffma2_rn(p, u, f2(0.05755210295319557f));
-    p = __ffma2_rn(p, u, f2(-0.0837731584906578f));
-    p = __ffma2_rn(p, u, f2(0.1094203069806099f));
-    p = __ffma2_rn(p, u, f2(-0.142619326710701f));
-    p = __ffma2_rn(p, u, f2(0.1999826580286026f));
-    p = __ffma2_rn(p, u, f2(-0.3333328366279602f));
+    float2 p = f2(kAtan9);
+    p = __ffma2_rn(p, u, f2(kAtan8));
+    p = __ffma2_rn(p, u, f2(kAtan7));
+    p = __ffma2_rn(p, u, f2(kAtan6));
+    p = __ffma2_rn(p, u, f2(kAtan5));
+    p = __ffma2_rn(p, u, f2(kAtan4));
+    p = __ffma2_rn(p, u, f2(kAtan3));
+    p = __ffma2_rn(p, u, f2(kAtan2));
+    p = __ffma2_rn(p, u, f2(kAtan1));
     p = __ffma2_rn(p, u, f2(1.0f));
     float2 r = __fmul2_rn(p, t);
     const float2 c = __fadd2_rn(neg2(r), f2(1.5707963267948966f));

@@ -476,6 +476,11 @@ __device__ __forceinline__ int reflect_idx(int i, int n) {
     return i >= n ? period - i : i;
 }
 
+// Coefficients of P below, by degree (wv_atan2 and its two-pixel form).
+constexpr float kAtan9 = -0.0017539301188662648f, kAtan8 = 0.010726944543421268f, kAtan7 = -0.030804596841335297f,
+                kAtan6 = 0.05755210295319557f, kAtan5 = -0.0837731584906578f, kAtan4 = 0.1094203069806099f,
+                kAtan3 = -0.142619326710701f, kAtan2 = 0.1999826580286026f, kAtan1 = -0.3333328366279602f;
+
 // atan2(y, x) in float32 for the projection, from a polynomial of this
 // library's own fit: atan(t) = t P(t^2) on [0, 1] with P of degree 9, the
 // coefficients minimising the largest relative error (Remez exchange; 2.4e-9
@@ -491,15 +496,15 @@ __device__ __forceinline__ float wv_atan2(float y, float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rcp) : "f"(mx));
     const float t = mx > 0.0f ? mn * rcp : 0.0f;
     const float u = t * t;
-    float p = -0.0017539301188662648f;
-    p = fmaf(p, u, 0.010726944543421268f);
-    p = fmaf(p, u, -0.030804596841335297f);
-    p = fmaf(p, u, 0.05755210295319557f);
-    p = fmaf(p, u, -0.0837731584906578f);
-    p = fmaf(p, u, 0.1094203069806099f);
-    p = fmaf(p, u, -0.142619326710701f);
-    p = fmaf(p, u, 0.1999826580286026f);
-    p = fmaf(p, u, -0.3333328366279602f);
+    float p = kAtan9;
+    p = fmaf(p, u, kAtan8);
+    p = fmaf(p, u, kAtan7);
+    p = fmaf(p, u, kAtan6);
+    p = fmaf(p, u, kAtan5);
+    p = fmaf(p, u, kAtan4);
+    p = fmaf(p, u, kAtan3);
+    p = fmaf(p, u, kAtan2);
+    p = fmaf(p, u, kAtan1);
     p = fmaf(p, u, 1.0f);
     float r = p * t;
     if (ay > ax) r = 1.5707963267948966f - r;

@@ -88,6 +88,7 @@ def test_batches_of_64_row_strips():
     w, h = 2048, 1024
     streams = [_stream(w, h, 5, 1, 1, False, 1), _stream(w, h, 5, 0, 1, False, 2), _stream(w, h, 4, 1, 0, False, 3),
                _stream(w, h, 3, 0, 0, False, 4)]
+
     def requests():
         rng = np.random.default_rng(7)
         out = []
