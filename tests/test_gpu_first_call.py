@@ -1,8 +1,8 @@
 """The first calls of a process: the kernels' code is loaded at their first use,
 which must not cost a player its first frames.  Opening a small stream and
 decoding its first viewport take 2.5 and 1.8 ms in a fresh process; with the
-device code compressed in the library they took 20 and 13.  The bounds lie at
-twice the former (best of three processes)."""
+device code compressed in the library they took 20 and 13.  The bounds lie below
+half of the latter (best of three processes, on machines of unequal hosts)."""
 import os
 import subprocess
 import sys
@@ -47,5 +47,5 @@ def test_first_open_and_first_viewport_of_a_process():
         assert r.returncode == 0, r.stderr[-4000:].decode()
         runs.append([float(v) for v in r.stdout.split()])
     opened, viewport = (min(c) for c in zip(*runs))
-    assert opened < 5.0, runs
-    assert viewport < 4.0, runs
+    assert opened < 9.0, runs
+    assert viewport < 6.0, runs
